@@ -18,7 +18,7 @@ constexpr int kDissQ = 5;
 constexpr int kDiss3Lat = 26;  // 3-D: 8 + 9 (G) + 9 (W) lattices of D3Q7
 constexpr int kDiss3Q = 7;
 
-template <class C> struct DissArgs {
+template <class C> struct DissArgs : RelaxTable<C, kDiss3Lat> {
     void *pop;
     int nx, ny, nz;
     int64_t stride;
@@ -28,6 +28,13 @@ template <class C> struct DissArgs {
     int powell;
     unsigned *flags;
 };
+
+// Relaxation constants of lattice k.
+template <int D> VLBM_HD __forceinline__ Relax<double> diss_relax(const DissArgs<double> &a, int k) { return a.relax[k]; }
+template <int D> VLBM_HD __forceinline__ Relax<float> diss_relax(const DissArgs<float> &a, int k)
+{
+    return relax_of<D, float>(a.omega[k]);
+}
 
 // Fluxes phi[k][c] along the two lattice axes and sources S[k] of one state.
 template <class C>

@@ -32,6 +32,7 @@
 // them and holds only the MHD lattices, forming each lattice's flux where it
 // relaxes that lattice (see k_diss3_step).
 #include "diss_cell.cuh"
+#include "ideal_cell.cuh"
 
 namespace vlbm {
 namespace {
@@ -92,19 +93,10 @@ __global__ void __launch_bounds__(kBlockX) k_diss_step(const DissArgs<C> a)
         C g[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) g[i] = HOLD ? f[HOLD ? k : 0][i] : *src(k, i);
-        const C om = a.omega[k];
-        const C omc = C(1) - om;
-        C ow0, ow1;
-        relax_weights<2, C>(om, ow0, ow1);
-        const C A0 = ow0 * q[k] + w0 * S[k];
-        const C A1 = ow1 * q[k] + w1 * S[k];
-        const C hom = C(0.5) * om;  // omega * w_moving / cs^2
-        const C bx = hom * phi[k][0], by = hom * phi[k][1];
-        *dst(k, 0) = omc * g[0] + A0;
-        *dst(k, 1) = omc * g[1] + A1 + bx;
-        *dst(k, 2) = omc * g[2] + A1 - bx;
-        *dst(k, 3) = omc * g[3] + A1 + by;
-        *dst(k, 4) = omc * g[4] + A1 - by;
+        const Relax<C> r = diss_relax<2>(a, k);
+        relax_lattice<2, C>(g, r, r.ow0 * q[k] + w0 * S[k], r.ow1 * q[k] + w1 * S[k], phi[k]);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) *dst(k, i) = g[i];
     }
 }
 
@@ -196,22 +188,11 @@ __device__ __forceinline__ void diss3_step_body(const DissArgs<C> &a)
     };
     constexpr C w0 = ExactWeights<3, C>::w0, w1 = ExactWeights<3, C>::w1;
     // BGK with direct source injection for lattice k, populations g, moment qk
-    auto relax = [&](int k, const C (&g)[Q], C qk, const C (&phi)[3], C S) {
-        const C om = a.omega[k];
-        const C omc = C(1) - om;
-        C ow0, ow1;
-        relax_weights<3, C>(om, ow0, ow1);
-        const C A0 = ow0 * qk + w0 * S;
-        const C A1 = ow1 * qk + w1 * S;
-        const C hom = C(0.5) * om;  // omega * w_moving / cs^2
-        const C bx = hom * phi[0], by = hom * phi[1], bz = hom * phi[2];
-        *dst(k, 0) = omc * g[0] + A0;
-        *dst(k, 1) = omc * g[1] + A1 + bx;
-        *dst(k, 2) = omc * g[2] + A1 - bx;
-        *dst(k, 3) = omc * g[3] + A1 + by;
-        *dst(k, 4) = omc * g[4] + A1 - by;
-        *dst(k, 5) = omc * g[5] + A1 + bz;
-        *dst(k, 6) = omc * g[6] + A1 - bz;
+    auto relax = [&](int k, C (&g)[Q], C qk, const C (&phi)[3], C S) {
+        const Relax<C> r = diss_relax<3>(a, k);
+        relax_lattice<3, C>(g, r, r.ow0 * qk + w0 * S, r.ow1 * qk + w1 * S, phi);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) *dst(k, i) = g[i];
     };
 
     // B's staging: pairs of gradient lattices, kNs stages of 14 populations per thread
@@ -475,7 +456,11 @@ template <class C> DissArgs<C> make_diss_args(vlbm_ctx *c)
     a.nz = d.nz;
     a.stride = d.stride;
     a.gm1 = C(d.gamma - 1.0);
-    for (int k = 0; k < kDiss3Lat; ++k) a.omega[k] = C(1.0 / (k < 8 ? d.tau[k] : p.tau_g));
+    for (int k = 0; k < kDiss3Lat; ++k) {
+        a.omega[k] = C(1.0 / (k < 8 ? d.tau[k] : p.tau_g));
+        if constexpr (sizeof(C) == 8)
+            a.relax[k] = c->dim == 2 ? relax_of<2, C>(a.omega[k]) : relax_of<3, C>(a.omega[k]);
+    }
     a.nu = C(p.nu);
     a.eta0 = C(p.eta0);
     a.inv_jc2 = C(p.j_c > 0.0 ? 1.0 / (p.j_c * p.j_c) : 0.0);

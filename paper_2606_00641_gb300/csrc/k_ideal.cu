@@ -20,7 +20,7 @@
 namespace vlbm {
 namespace {
 
-template <class C> struct IdealArgs {
+template <class C> struct IdealArgs : RelaxTable<C, kMaxLat> {
     void *pop;
     int nx, ny, nz;
     int64_t stride;
@@ -39,6 +39,10 @@ template <class C> struct IdealArgs {
     const double *refscale;  // deviation storage: r_0..7, s_0..7 in FP64 (device; pressure recovery)
     C p_theta;               // deviation storage: FP64 pressure below p_theta * e_tot
 };
+
+// What a step's collision takes its relaxation constants from.
+__device__ __forceinline__ const RelaxTable<double, kMaxLat> &step_omega(const IdealArgs<double> &a) { return a; }
+__device__ __forceinline__ const float *step_omega(const IdealArgs<float> &a) { return a.omega; }
 
 // Linear indices of the cell's neighbours x + c_i (periodic), i in set order.
 template <int D>
@@ -59,6 +63,15 @@ __device__ __forceinline__ void neighbours(int x, int y, int z, int nx, int ny, 
     }
 }
 
+
+// The n-th direction of a loop over one lattice's slots.  FP64 walks the slots in
+// memory order (SWAP: the loop's slot is opp(i)); in direction order the compiler
+// added 34 register moves a cell to the FP64 pipe, which binds that step (2-D: 205
+// FP64 instructions a cell, 169 in memory order).
+template <class C, bool SWAP> __device__ __forceinline__ constexpr int slot_order(int n)
+{
+    return sizeof(C) == 8 && SWAP ? opp_axis(n) : n;
+}
 
 // The fused collide-and-stream step.  ODD selects the AA parity; CORR adds
 // the learned flux correction dPhi[k][a] to the post-collision populations
@@ -82,24 +95,27 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
 #pragma unroll
     for (int k = 0; k < NL; ++k)
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
+        for (int n = 0; n < Q; ++n) {
+            const int i = slot_order<C, ODD>(n);
             const int j = ODD ? opp_axis(i) : i;
             const int64_t at = ODD ? nb[opp_axis(i)] : cell;
             f[k][i] = Codec<S>::load(pop + (int64_t)(k * Q + j) * a.stride + at);
         }
 
+    const auto &omega = step_omega(a);
     if constexpr (NL == 9) {
-        powell_collide<D, C>(f, a.gm1, a.omega, a.src0, a.src1, a.inv_tau_m, a.flags);
+        powell_collide<D, C>(f, a.gm1, omega, a.src0, a.src1, a.inv_tau_m, a.flags);
     } else if constexpr (HOM) {
         const float *sp = a.solid + cell;
         const C d = C(__ldg(sp));
         const C uB[3] = {C(__ldg(sp + a.solid_n)), C(__ldg(sp + 2 * a.solid_n)), C(__ldg(sp + 3 * a.solid_n))};
         const C BB[3] = {C(__ldg(sp + 4 * a.solid_n)), C(__ldg(sp + 5 * a.solid_n)), C(__ldg(sp + 6 * a.solid_n))};
-        ideal_collide_hom<D, C>(f, a.gm1, a.omega, a.src0, a.src1, a.flags, d, uB, BB);
+        ideal_collide_hom<D, C>(f, a.gm1, omega, a.src0, a.src1, a.flags, d, uB, BB);
     } else {
         // deviation storage collides on the stored deviations directly (ideal_cell.cuh)
-        ideal_collide<D, C, Codec<S>::kDev>(f, a.gm1, a.omega, a.src0, a.src1, a.flags, a.ref, a.scale,
-                                            a.inv_scale, a.refscale, a.p_theta);
+        if constexpr (sizeof(C) == 8) ideal_collide_f64<D, C>(f, a.gm1, omega, a.src0, a.src1, a.flags);
+        else ideal_collide<D, C, Codec<S>::kDev>(f, a.gm1, a.omega, a.src0, a.src1, a.flags, a.ref, a.scale,
+                                                 a.inv_scale, a.refscale, a.p_theta);
     }
     if constexpr (CORR) {
         const float *dp = a.dphi + cell * 24;
@@ -118,7 +134,8 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
 #pragma unroll
     for (int k = 0; k < NL; ++k)
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
+        for (int n = 0; n < Q; ++n) {
+            const int i = slot_order<C, !ODD>(n);
             const int j = ODD ? i : opp_axis(i);
             const int64_t at = ODD ? nb[i] : cell;
             Codec<S>::store(pop + (int64_t)(k * Q + j) * a.stride + at, f[k][i]);
@@ -780,12 +797,14 @@ template <class C> IdealArgs<C> make_step_args(vlbm_ctx *c)
     const bool dev = c->storage == VLBM_F16_DEV || c->storage == VLBM_BF16_DEV;
     for (int k = 0; k < kMaxLat; ++k) {
         const double s = dev ? d.q_scale[k] : 1.0;
-        a.omega[k] = C(1.0 / d.tau[k]);
         a.src0[k] = C(w0 * d.source[k] / s);
         a.src1[k] = C(w1 * d.source[k] / s);
         a.ref[k] = C(dev ? d.q_ref[k] : 0.0);
         a.scale[k] = C(s);
         a.inv_scale[k] = C(1.0 / s);
+        a.omega[k] = C(1.0 / d.tau[k]);
+        if constexpr (sizeof(C) == 8)
+            a.relax[k] = c->dim == 2 ? relax_of<2, C>(a.omega[k]) : relax_of<3, C>(a.omega[k]);
     }
     a.flags = c->d_flags;
     a.inv_tau_m = C(1.0 / d.tau_m);

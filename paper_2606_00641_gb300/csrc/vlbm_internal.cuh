@@ -101,6 +101,42 @@ template <int D, class C> VLBM_HD __forceinline__ void relax_weights(C om, C &ow
     ow0 = D == 2 ? om - C(4) * ow1 : om * ExactWeights<D, C>::w0;
 }
 
+// Relaxation constants of one lattice: 1 - omega, omega w_0, omega w_moving and
+// omega w_moving / cs^2.
+template <class C> struct Relax {
+    C omc, ow0, ow1, hom;
+};
+
+// The same for N lattices, worked out once on the host and passed as kernel
+// parameters, so that an FP64 collision reads them as constant operands.  Formed
+// from omega in every thread instead they were five operations per lattice and
+// cell, the same for all cells: 40 of the 240 FP64 instructions of a D2Q5 cell
+// (the FP64 pipe binds that kernel).  FP32 kernels, which HBM binds, form them from
+// omega; their parameters hold no table.
+template <class C, int N> struct RelaxTable {};
+template <int N> struct RelaxTable<double, N> {
+    Relax<double> relax[N];
+};
+
+template <int D, class C> VLBM_HD __forceinline__ Relax<C> relax_of(C om)
+{
+    Relax<C> r;
+    r.omc = C(1) - om;
+    relax_weights<D, C>(om, r.ow0, r.ow1);
+    r.hom = C(0.5) * om;
+    return r;
+}
+
+// The constants of lattice k from the table, or worked out from omega[k].
+template <int D, int N> VLBM_HD __forceinline__ Relax<double> relax_at(const RelaxTable<double, N> &t, int k)
+{
+    return t.relax[k];
+}
+template <int D, class C> VLBM_HD __forceinline__ Relax<C> relax_at(const C *omega, int k)
+{
+    return relax_of<D, C>(omega[k]);
+}
+
 // An opaque copy of a value: the compiler cannot reuse expressions computed
 // from the original across it, so addresses built from the copy are
 // recomputed where they are used instead of being held in registers.
