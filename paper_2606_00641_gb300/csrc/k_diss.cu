@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kBlockX) k_diss_step(const DissArgs<C> a)
             s += v;
         }
         q[k] = s;
+        keep_f64(q[k]);
     }
     C phi[kDissLat][2], S[kDissLat];
     diss_flux_source<C>(q, a, phi, S, a.flags);

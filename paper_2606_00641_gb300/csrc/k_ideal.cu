@@ -65,9 +65,9 @@ __device__ __forceinline__ void neighbours(int x, int y, int z, int nx, int ny, 
 
 
 // The n-th direction of a loop over one lattice's slots.  FP64 walks the slots in
-// memory order (SWAP: the loop's slot is opp(i)); in direction order the compiler
-// added 34 register moves a cell to the FP64 pipe, which binds that step (2-D: 205
-// FP64 instructions a cell, 169 in memory order).
+// memory order (SWAP: the loop's slot is opp(i)): with the even parity's stores in
+// direction order the compiler put some 40 more operations a cell on the FP64 pipe,
+// which binds that step.
 template <class C, bool SWAP> __device__ __forceinline__ constexpr int slot_order(int n)
 {
     return sizeof(C) == 8 && SWAP ? opp_axis(n) : n;
