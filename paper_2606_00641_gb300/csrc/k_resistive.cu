@@ -20,18 +20,15 @@
 // of the same direction -- the halfway bounce-back in AA form.
 #include "vlbm_internal.cuh"
 
+#include "split_f32.cuh"
+
 namespace vlbm {
 namespace {
 
 constexpr int kQf = 19;
 constexpr int kSlots = 19 + 21;
 
-// D3Q19 velocities in the ABI order; opposite of i is opp_axis(i).
-__constant__ signed char c19[kQf][3] = {
-    {0, 0, 0},   {1, 0, 0},   {-1, 0, 0}, {0, 1, 0},  {0, -1, 0}, {0, 0, 1},  {0, 0, -1},
-    {1, 1, 0},   {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0}, {1, 0, 1},  {-1, 0, -1}, {1, 0, -1},
-    {-1, 0, 1},  {0, 1, 1},   {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
-
+// D3Q19 velocities in the ABI order: i = 2 p - 1 and 2 p are opposite (opp_axis).
 __host__ __device__ constexpr int cx19(int i)
 {
     return (i == 1 || i == 7 || i == 9 || i == 11 || i == 13) ? 1
@@ -228,49 +225,125 @@ __global__ void __launch_bounds__(kBlockX, 5) k_res_step(const Args a)
         }
 }
 
-// f = f_eq(rho, m - F/2, B), g = g_eq(B, u = m/rho) at parity 0, in double.
+// f = f_eq(rho, m - F/2, B), g = g_eq(B, u = m/rho) at parity 0, rounded to FP32 once.
+// Carried in split floats (split_f32.cuh): in FP64, with the velocities in a table, the
+// pass took 4.22 ms at 128 x 128 x 256 for 0.13 ms worth of memory traffic; 0.49 ms so.  Opposite
+// directions share the part even in c, w (rho + 4.5 (c c - cs2 I):(rho v v + ...)), and
+// differ in the sign of the odd one, 3 w c.j.
 struct InitArgs {
     float *pop;
     int64_t stride, c0, count, qstride;
     double F[3];
 };
 
-__global__ void k_res_init(const InitArgs a, const double *__restrict__ Qin)
+// The same in FP64, for states beyond the range in which split floats keep their digits.
+__device__ __noinline__ void res_init_wide(const InitArgs &a, const double *__restrict__ Qin, int64_t t, float *out)
 {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= a.count) return;
-    const int64_t cell = a.c0 + t;
     const double rho = Qin[t];
-    double m[3], j[3], B[3], u[3];
+    double m[3], j[3], B[3], u[3], v[3];
     for (int ax = 0; ax < 3; ++ax) {
         m[ax] = Qin[(1 + ax) * a.qstride + t];
         B[ax] = Qin[(4 + ax) * a.qstride + t];
         j[ax] = m[ax] - 0.5 * a.F[ax];
         u[ax] = m[ax] / rho;
+        v[ax] = j[ax] / rho;
     }
-    const double v[3] = {j[0] / rho, j[1] / rho, j[2] / rho};
     const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
     const double B2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
+#pragma unroll 1
     for (int i = 0; i < kQf; ++i) {
-        const double cv = c19[i][0] * v[0] + c19[i][1] * v[1] + c19[i][2] * v[2];
-        const double cj = c19[i][0] * j[0] + c19[i][1] * j[1] + c19[i][2] * j[2];
-        const double cB = c19[i][0] * B[0] + c19[i][1] * B[1] + c19[i][2] * B[2];
-        const double c2 = c19[i][0] * c19[i][0] + c19[i][1] * c19[i][1] + c19[i][2] * c19[i][2];
+        const int c[3] = {cx19(i), cy19(i), cz19(i)};
+        const double cv = c[0] * v[0] + c[1] * v[1] + c[2] * v[2];
+        const double cj = c[0] * j[0] + c[1] * j[1] + c[2] * j[2];
+        const double cB = c[0] * B[0] + c[1] * B[1] + c[2] * B[2];
+        const double c2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
         const double second = rho * (cv * cv - v2 / 3.0) + 0.5 * B2 * (c2 - 1.0) - (cB * cB - B2 / 3.0);
         const double w = i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
-        a.pop[(int64_t)i * a.stride + cell] = (float)(w * (rho + 3.0 * cj + 4.5 * second));
+        out[(int64_t)i * a.stride] = (float)(w * (rho + 3.0 * cj + 4.5 * second));
     }
-    for (int b = 0; b < 3; ++b)
-        for (int i = 0; i < 7; ++i) {
-            double cphi = 0.0;
-            if (i > 0) {
-                const int ax = (i - 1) / 2;
-                const double s = (i & 1) ? 1.0 : -1.0;
-                cphi = (ax == b) ? 0.0 : s * (u[ax] * B[b] - B[ax] * u[b]);
-            }
-            const double w = i == 0 ? 0.25 : 0.125;
-            a.pop[(int64_t)(19 + 7 * b + i) * a.stride + cell] = (float)(w * (B[b] + 4.0 * cphi));
+#pragma unroll 1
+    for (int i = 0; i < 21; ++i) {
+        const int b = i / 7, d = i % 7, ax = (d - 1) / 2;
+        double cphi = 0.0;
+        if (d > 0 && ax != b) cphi = ((d & 1) ? 1.0 : -1.0) * (u[ax] * B[b] - B[ax] * u[b]);
+        out[(int64_t)(kQf + i) * a.stride] = (float)((d == 0 ? 0.25 : 0.125) * (B[b] + 4.0 * cphi));
+    }
+}
+
+__global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double *__restrict__ Qin)
+{
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= a.count) return;
+    float *out = a.pop + a.c0 + t;
+    {
+        bool usual = Qin[t] > 1e-6 && Qin[t] < 1e6;
+#pragma unroll
+        for (int k = 1; k < 7; ++k) usual = usual && fabs(Qin[k * a.qstride + t]) < 1e6;
+        if (!usual) {
+            res_init_wide(a, Qin, t, out);
+            return;
         }
+    }
+    const Split rho = split(Qin[t]);
+    Split j[3], B[3], u[3], v[3];
+    const Split ir = reciprocal(rho);
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        const double m = Qin[(1 + ax) * a.qstride + t];
+        B[ax] = split(Qin[(4 + ax) * a.qstride + t]);
+        j[ax] = split(m - 0.5 * a.F[ax]);
+        u[ax] = split(m) * ir;
+        v[ax] = j[ax] * ir;
+    }
+    const Split third = {1.f / 3.f, (float)(1.0 / 3.0 - (double)(1.f / 3.f))};
+    const Split B2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
+    const Split v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    // (c c - cs2 I) : (rho v v + B^2/2 I - B B) = rho (c.v)^2 - (c.B)^2 + (c^2 - 1) B^2/2 + base
+    const Split base = (B2 - rho * v2) * third;
+    const Split four_half = {4.5f, 0.f}, three = {3.f, 0.f}, halfs = {0.5f, 0.f};
+    const Split hB2 = halfs * B2;
+#pragma unroll
+    for (int p = 0; p < 10; ++p) {  // the rest population, then the nine opposite pairs
+        const int i = p == 0 ? 0 : 2 * p - 1;
+        const double wd = i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
+        const Split w = {(float)wd, (float)(wd - (double)(float)wd)};
+        auto along = [&](const Split (&x)[3]) {  // c_i . x, i a compile-time constant
+            Split s = {0.f, 0.f};
+            bool first = true;
+            const int c[3] = {cx19(i), cy19(i), cz19(i)};
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax)
+                if (c[ax] != 0) {
+                    const Split y = c[ax] > 0 ? x[ax] : -x[ax];
+                    s = first ? y : s + y;
+                    first = false;
+                }
+            return s;
+        };
+        if (p == 0) {
+            out[0] = (w * (rho + four_half * (base - hB2))).hi;
+            continue;
+        }
+        const Split cv = along(v), cB = along(B);
+        Split second = base + rho * (cv * cv) - cB * cB;
+        if (i > 6) second = second + hB2;
+        const Split even = w * (rho + four_half * second), odd = w * (three * along(j));
+        out[(int64_t)i * a.stride] = (even + odd).hi;
+        out[(int64_t)(i + 1) * a.stride] = (even - odd).hi;
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        float *g = out + (int64_t)(kQf + 7 * b) * a.stride;
+        g[0] = 0.25f * B[b].hi;
+        const Split w = {0.125f, 0.f}, B8 = w * B[b];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {  // w (B +- 4 (u_a B_b - B_a u_b)), zero for a = b
+            Split s = {0.f, 0.f};
+            if (ax != b) s = halfs * (u[ax] * B[b] - B[ax] * u[b]);
+            g[(int64_t)(2 * ax + 1) * a.stride] = (B8 + s).hi;
+            g[(int64_t)(2 * ax + 2) * a.stride] = (B8 - s).hi;
+        }
+    }
 }
 
 struct ReadArgs {
@@ -307,41 +380,95 @@ __device__ double res_logical(const ReadArgs &a, int64_t cell, int x, int y, int
     return a.pop[(int64_t)(19 + 7 * b + opp_axis(i)) * a.stride + nbr(o, cell, -cx19(i), -cy19(i), -cz19(i))];
 }
 
-__device__ void res_cell_moments(const ReadArgs &a, int64_t cell, double *q)
+// Moments of one cell in FP64 from its FP32 populations: sums carried in three floats
+// (split_f32.cuh), the 40 conversions and 110 additions of the FP64 form on the slow
+// FP64 pipe replaced (1.55 -> 0.29 ms a pass at 128 x 128 x 256, 0.13 ms of it memory
+// traffic).  A sum that leaves the finite numbers is formed again in FP64.
+template <bool ODD>
+__device__ __forceinline__ void res_cell_moments(const ReadArgs &a, int64_t cell, double (&q)[7])
 {
     int x, y, z;
     cell_xyz(cell, a.nx, a.ny, x, y, z);
     if (wall_row(y, a.ny, a.walls_y)) {
         q[0] = 1.0;
+#pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
             q[1 + ax] = 0.0;
             q[4 + ax] = a.bw[ax];
         }
         return;
     }
-    double rho = 0, m[3] = {0, 0, 0}, B[3] = {0, 0, 0};
+    const Offsets o = offsets(x, y, z, a.nx, a.ny, a.nz);
+    const bool wall_lo = a.walls_y && y == 1, wall_hi = a.walls_y && y == a.ny - 2;
+    auto flow = [&](int i) -> float {
+        if (!ODD) return a.pop[(int64_t)i * a.stride + cell];
+        const bool from_wall = (cy19(i) > 0 && wall_lo) || (cy19(i) < 0 && wall_hi);
+        const int64_t at = from_wall ? cell : nbr(o, cell, -cx19(i), -cy19(i), -cz19(i));
+        return a.pop[(int64_t)(from_wall ? i : opp_axis(i)) * a.stride + at];
+    };
+    auto magnetic = [&](int b, int i) -> float {
+        if (!ODD) return a.pop[(int64_t)(kQf + 7 * b + i) * a.stride + cell];
+        return a.pop[(int64_t)(kQf + 7 * b + opp_axis(i)) * a.stride + nbr(o, cell, -cx19(i), -cy19(i), -cz19(i))];
+    };
+    Sum3 s[7];
+    float f[kQf];
+#pragma unroll
+    for (int i = 0; i < kQf; ++i) f[i] = flow(i);
+#pragma unroll
     for (int i = 0; i < kQf; ++i) {
-        const double v = res_logical(a, cell, x, y, z, i);
-        rho += v;
-        m[0] += c19[i][0] * v;
-        m[1] += c19[i][1] * v;
-        m[2] += c19[i][2] * v;
+        s[0].add(f[i]);
+        const int c[3] = {cx19(i), cy19(i), cz19(i)};
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax)
+            if (c[ax] != 0) s[1 + ax].add(c[ax] > 0 ? f[i] : -f[i]);
     }
-    for (int b = 0; b < 3; ++b)
-        for (int i = 0; i < 7; ++i) B[b] += res_logical(a, cell, x, y, z, kQf + 7 * b + i);
-    q[0] = rho;
-    for (int ax = 0; ax < 3; ++ax) {
-        q[1 + ax] = m[ax] + 0.5 * a.F[ax];
-        q[4 + ax] = B[ax];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        float g[7];
+#pragma unroll
+        for (int i = 0; i < 7; ++i) g[i] = magnetic(b, i);
+#pragma unroll
+        for (int i = 0; i < 7; ++i) s[4 + b].add(g[i]);
     }
+    bool finite = true;
+#pragma unroll
+    for (int v = 0; v < 7; ++v) {
+        finite = finite && s[v].finite();
+        q[v] = s[v].value();
+    }
+    if (!finite) {
+        double d[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+        for (int i = 0; i < kQf; ++i) {
+            const double v = res_logical(a, cell, x, y, z, i);
+            d[0] += v;
+            d[1] += cx19(i) * v;
+            d[2] += cy19(i) * v;
+            d[3] += cz19(i) * v;
+        }
+#pragma unroll 1
+        for (int i = 0; i < 21; ++i) {
+            const double v = res_logical(a, cell, x, y, z, kQf + i);
+            if (i < 7) d[4] += v;
+            else if (i < 14) d[5] += v;
+            else d[6] += v;
+        }
+#pragma unroll
+        for (int v = 0; v < 7; ++v) q[v] = d[v];
+    }
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) q[1 + ax] += 0.5 * a.F[ax];
 }
 
-__global__ void k_res_moments(const ReadArgs a, int64_t c0, int64_t count, int64_t ostride, double *__restrict__ out)
+template <bool ODD>
+__global__ void __launch_bounds__(128) k_res_moments(const ReadArgs a, int64_t c0, int64_t count, int64_t ostride,
+                                                     double *__restrict__ out)
 {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= count) return;
     double q[7];
-    res_cell_moments(a, c0 + t, q);
+    res_cell_moments<ODD>(a, c0 + t, q);
+#pragma unroll
     for (int v = 0; v < 7; ++v) out[v * ostride + t] = q[v];
 }
 
@@ -355,6 +482,7 @@ __global__ void k_res_gather(const ReadArgs a, const int64_t *__restrict__ cells
     for (int j = 0; j < kSlots; ++j) out[(int64_t)t * kSlots + j] = res_logical(a, cell, x, y, z, j);
 }
 
+template <bool ODD>
 __global__ void __launch_bounds__(kReduceThreads) k_res_partials(const ReadArgs a, int64_t ncell,
                                                                  double *__restrict__ partials)
 {
@@ -362,23 +490,11 @@ __global__ void __launch_bounds__(kReduceThreads) k_res_partials(const ReadArgs 
     for (int64_t cell = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; cell < ncell;
          cell += (int64_t)gridDim.x * blockDim.x) {
         double q[7];
-        res_cell_moments(a, cell, q);
+        res_cell_moments<ODD>(a, cell, q);
+#pragma unroll
         for (int v = 0; v < 7; ++v) acc[v] += q[v];
     }
-    __shared__ double red[kReduceThreads / 32][8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int v = 0; v < 7; ++v) {
-        double s = acc[v];
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (lane == 0) red[warp][v] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        double s = 0.0;
-        if (threadIdx.x < 7)
-            for (int w = 0; w < kReduceThreads / 32; ++w) s += red[w][threadIdx.x];
-        partials[(int64_t)blockIdx.x * 8 + threadIdx.x] = s;
-    }
+    write_partial(acc, partials);
 }
 
 Args make_args(vlbm_ctx *c)
@@ -445,7 +561,7 @@ vlbm_status resistive_init_range(vlbm_ctx *c, int di, const double *Q, int64_t c
     a.count = n;
     a.qstride = qstride;
     for (int ax = 0; ax < 3; ++ax) a.F[ax] = d.force[ax];
-    k_res_init<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(a, Q);
+    k_res_init<<<(unsigned)((n + 127) / 128), 128, 0, c->stream>>>(a, Q);
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "resistive init launch");
 }
@@ -458,7 +574,10 @@ vlbm_status resistive_init(vlbm_ctx *c, int d, const double *Q_dev)
 
 vlbm_status resistive_moments_range(vlbm_ctx *c, int di, double *out, int64_t c0, int64_t n, int64_t ostride)
 {
-    k_res_moments<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(make_read(c, di), c0, n, ostride, out);
+    const ReadArgs a = make_read(c, di);
+    const unsigned blocks = (unsigned)((n + 127) / 128);
+    if (a.parity) k_res_moments<true><<<blocks, 128, 0, c->stream>>>(a, c0, n, ostride, out);
+    else k_res_moments<false><<<blocks, 128, 0, c->stream>>>(a, c0, n, ostride, out);
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "resistive moments launch");
 }
@@ -478,12 +597,15 @@ vlbm_status resistive_gather(vlbm_ctx *c, int di, const int64_t *cells_dev, int 
 
 vlbm_status resistive_sums(vlbm_ctx *c, int di, double *sums_dev)
 {
-    k_res_partials<<<kReduceBlocks, kReduceThreads, 0, c->stream>>>(make_read(c, di), c->dom[di].ncell,
-                                                                    c->d_partials);
+    const ReadArgs a = make_read(c, di);
+    const int64_t ncell = c->dom[di].ncell;
+    const int blocks = reduce_blocks(ncell);
+    if (a.parity) k_res_partials<true><<<blocks, kReduceThreads, 0, c->stream>>>(a, ncell, c->d_partials);
+    else k_res_partials<false><<<blocks, kReduceThreads, 0, c->stream>>>(a, ncell, c->d_partials);
     c->launches++;
     vlbm_status s = cuda_check(c, cudaGetLastError(), "resistive partial sums launch");
     if (s != VLBM_OK) return s;
-    return finish_sums(c, 7, sums_dev);
+    return finish_sums(c, blocks, 7, sums_dev);
 }
 
 }  // namespace vlbm

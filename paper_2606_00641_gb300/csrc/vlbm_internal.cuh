@@ -191,6 +191,38 @@ template <> struct ComputeOf<double> {
     using T = double;
 };
 
+// CTAs of a domain-sum pass: one cell a thread up to kReduceBlocks CTAs.  A CTA's last
+// act, adding its threads' eight sums, costs 40 FP64 additions a warp on a pipe that
+// takes 16 cycles each, so a small domain is not spread over CTAs without cells:
+// 30,000 cells took 31 us with all kReduceBlocks CTAs, 8 with 118.
+inline int reduce_blocks(int64_t ncell)
+{
+    const int64_t need = (ncell + kReduceThreads - 1) / kReduceThreads;
+    return (int)(need < 1 ? 1 : need < kReduceBlocks ? need : kReduceBlocks);
+}
+
+// The CTA's sum of its threads' NV values into its row of eight partials (zeros beyond
+// NV): shuffles within the warps, then one thread per value over the warps.
+template <int NV> __device__ __forceinline__ void write_partial(const double (&acc)[NV], double *__restrict__ partials)
+{
+    __shared__ double red[kReduceThreads / 32][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        double v = acc[k];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0) red[warp][k] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double v = 0.0;
+        if (threadIdx.x < NV)
+            for (int w = 0; w < kReduceThreads / 32; ++w) v += red[w][threadIdx.x];
+        partials[(int64_t)blockIdx.x * 8 + threadIdx.x] = v;
+    }
+}
+
 // Per-domain description (host and device copies).
 struct Domain {
     int nx, ny, nz;
@@ -360,6 +392,6 @@ HaloSlots halo_slots(const vlbm_ctx *c);
 vlbm_status halo_copy(vlbm_ctx *c, void *lo, void *hi, bool pack);
 
 // reduction of per-block partials into sums (k_ideal.cu)
-vlbm_status finish_sums(vlbm_ctx *c, int nvar, double *sums_dev);
+vlbm_status finish_sums(vlbm_ctx *c, int blocks, int nvar, double *sums_dev);
 
 }  // namespace vlbm
