@@ -27,6 +27,7 @@ template <class C> struct DissArgs : RelaxTable<C, kDiss3Lat> {
     C nu, eta0, inv_jc2, inv_tau_m;
     int powell;
     unsigned *flags;
+    FastDiv by_nx;
 };
 
 // Relaxation constants of lattice k.

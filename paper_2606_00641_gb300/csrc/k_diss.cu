@@ -52,13 +52,12 @@ __device__ __forceinline__ void diss_neighbours(int x, int y, int nx, int ny, in
 // sends direction i to slot (opp i, x); odd parity reads slot (opp i, x - c_i)
 // and sends direction i to slot (i, x + c_i).  HOLD keeps the populations in
 // registers between load and update, otherwise they are read twice.
-template <class C, bool ODD, bool HOLD>
+template <class C, bool ODD, bool HOLD, bool PLANES>
 __global__ void __launch_bounds__(kBlockX) k_diss_step(const DissArgs<C> a)
 {
     constexpr int Q = kDissQ;
-    const int x = blockIdx.x * kBlockX + threadIdx.x;
-    if (x >= a.nx) return;
-    const int y = blockIdx.y;
+    int x, y, z;
+    if (!step_cell<PLANES>(a.nx, a.ny, a.by_nx, x, y, z)) return;
     const int64_t cell = x + (int64_t)a.nx * y;
     int64_t nb[Q];
     diss_neighbours(x, y, a.nx, a.ny, cell, nb);
@@ -170,13 +169,12 @@ __device__ __forceinline__ void diss3_neighbours(int x, int y, int z, int nx, in
 // into L2 at its start; 3.37 with the MHD lattices staged too, at four CTAs per
 // SM).  FP64 (HOLD false) keeps nothing in registers and reads the MHD lattices
 // again in C (the FP64 pipe binds that form, not the memory traffic).
-template <class C, bool ODD, bool HOLD>
+template <class C, bool ODD, bool HOLD, bool PLANES>
 __device__ __forceinline__ void diss3_step_body(const DissArgs<C> &a)
 {
     constexpr int Q = kDiss3Q;
-    const int x = blockIdx.x * kBlockX + threadIdx.x;
-    if (x >= a.nx) return;
-    const int y = blockIdx.y, z = blockIdx.z;
+    int x, y, z;
+    if (!step_cell<PLANES>(a.nx, a.ny, a.by_nx, x, y, z)) return;
     const int64_t cell = x + (int64_t)a.nx * (y + (int64_t)a.ny * z);
     int64_t nb[Q];
     diss3_neighbours(x, y, z, a.nx, a.ny, a.nz, cell, nb);
@@ -295,10 +293,10 @@ __device__ __forceinline__ void diss3_step_body(const DissArgs<C> &a)
 
 // Three CTAs of the FP32 form fit an SM at 168 registers and 28 KB of staging each
 // (the FP64 form keeps the compiler's own register choice)
-template <class C, bool ODD, bool HOLD>
+template <class C, bool ODD, bool HOLD, bool PLANES>
 __global__ void __launch_bounds__(kBlockX, HOLD ? 3 : 0) k_diss3_step(const DissArgs<C> a)
 {
-    diss3_step_body<C, ODD, HOLD>(a);
+    diss3_step_body<C, ODD, HOLD, PLANES>(a);
 }
 
 // 3-D f = f_eq(Q) at parity 0, and the positivity and sub-characteristic checks.
@@ -481,18 +479,14 @@ template <class C> vlbm_status step_t(vlbm_ctx *c, int parity)
 {
     constexpr bool hold = sizeof(C) == 4;
     const Domain &d = c->dom[0];
-    const DissArgs<C> a = make_diss_args<C>(c);
-    const dim3 grid((unsigned)((d.nx + kBlockX - 1) / kBlockX), (unsigned)d.ny, (unsigned)d.nz);
-    if (c->dim == 3) {
-        if (parity)
-            k_diss3_step<C, true, hold><<<grid, kBlockX, 0, c->stream>>>(a);
-        else
-            k_diss3_step<C, false, hold><<<grid, kBlockX, 0, c->stream>>>(a);
-    } else if (parity) {
-        k_diss_step<C, true, hold><<<grid, kBlockX, 0, c->stream>>>(a);
-    } else {
-        k_diss_step<C, false, hold><<<grid, kBlockX, 0, c->stream>>>(a);
-    }
+    DissArgs<C> a = make_diss_args<C>(c);
+    const StepGrid g = step_grid(d.nx, d.ny, d.nz);
+    a.by_nx = g.nx;
+    with_flags(parity != 0, g.planes, [&](auto odd, auto planes) {
+        constexpr bool O = decltype(odd)::value, P = decltype(planes)::value;
+        if (c->dim == 3) k_diss3_step<C, O, hold, P><<<g.grid, kBlockX, 0, c->stream>>>(a);
+        else k_diss_step<C, O, hold, P><<<g.grid, kBlockX, 0, c->stream>>>(a);
+    });
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "dissipative step launch");
 }

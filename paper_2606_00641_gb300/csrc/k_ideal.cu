@@ -38,6 +38,7 @@ template <class C> struct IdealArgs : RelaxTable<C, kMaxLat> {
     int64_t solid_n;
     const double *refscale;  // deviation storage: r_0..7, s_0..7 in FP64 (device; pressure recovery)
     C p_theta;               // deviation storage: FP64 pressure below p_theta * e_tot
+    FastDiv by_nx;
 };
 
 // What a step's collision takes its relaxation constants from.
@@ -78,13 +79,12 @@ template <class C, bool SWAP> __device__ __forceinline__ constexpr int slot_orde
 // (f*_{k,+a} += dPhi/2, f*_{k,-a} -= dPhi/2: zero mass, first moment dPhi).
 // NL = 9 is the Powell model (eight MHD lattices and the divergence lattice);
 // HOM blends with homogenised solids (a.solid).
-template <int D, class S, class C, bool ODD, bool CORR = false, int NL = 8, bool HOM = false>
+template <int D, class S, class C, bool ODD, bool CORR, int NL, bool HOM, bool PLANES>
 __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
 {
     constexpr int Q = AxisSet<D>::Q;
-    const int x = blockIdx.x * kBlockX + threadIdx.x;
-    if (x >= a.nx) return;
-    const int y = blockIdx.y, z = blockIdx.z;
+    int x, y, z;
+    if (!step_cell<PLANES>(a.nx, a.ny, a.by_nx, x, y, z)) return;
     const int64_t cell = x + (int64_t)a.nx * (y + (int64_t)a.ny * z);
     int64_t nb[Q];
     neighbours<D>(x, y, z, a.nx, a.ny, a.nz, cell, nb);
@@ -142,19 +142,19 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
         }
 }
 
-template <int D, class S, class C, bool ODD, bool CORR = false, int NL = 8, bool HOM = false>
+template <int D, class S, class C, bool ODD, bool PLANES, bool CORR = false, int NL = 8, bool HOM = false>
 __global__ void __launch_bounds__(kBlockX) k_ideal_step(const IdealArgs<C> a)
 {
-    ideal_step_body<D, S, C, ODD, CORR, NL, HOM>(a);
+    ideal_step_body<D, S, C, ODD, CORR, NL, HOM, PLANES>(a);
 }
 
 // Deviation storage: the same step bounded to the occupancy of the plain 16-bit
 // step (six CTAs per SM in 2-D, five in 3-D), so that the rare FP64
 // pressure-recovery call does not lower it.
-template <int D, class S, bool ODD>
+template <int D, class S, bool ODD, bool PLANES>
 __global__ void __launch_bounds__(kBlockX, D == 2 ? 6 : 5) k_ideal_step_dev(const IdealArgs<float> a)
 {
-    ideal_step_body<D, S, float, ODD>(a);
+    ideal_step_body<D, S, float, ODD, false, 8, false, PLANES>(a);
 }
 
 // The same step for 16-bit storage in 3-D with the loads done by the
@@ -823,26 +823,7 @@ template <int D, class S> ReadArgs<D, S> make_read_args(vlbm_ctx *c, int di)
 template <int D, class S, class C> vlbm_status step_t(vlbm_ctx *c, int parity)
 {
     const Domain &d = c->dom[0];
-    const IdealArgs<C> a = make_step_args<C>(c);
-    const dim3 grid((unsigned)((d.nx + kBlockX - 1) / kBlockX), (unsigned)d.ny, (unsigned)d.nz);
-    if constexpr (!Codec<S>::kDev) {
-        if (c->solid) {  // homogenised solids
-            if (parity)
-                k_ideal_step<D, S, C, true, false, 8, true><<<grid, kBlockX, 0, c->stream>>>(a);
-            else
-                k_ideal_step<D, S, C, false, false, 8, true><<<grid, kBlockX, 0, c->stream>>>(a);
-            c->launches++;
-            return cuda_check(c, cudaGetLastError(), "homogenised step launch");
-        }
-        if (c->nlat == 9) {  // Powell model
-            if (parity)
-                k_ideal_step<D, S, C, true, false, 9><<<grid, kBlockX, 0, c->stream>>>(a);
-            else
-                k_ideal_step<D, S, C, false, false, 9><<<grid, kBlockX, 0, c->stream>>>(a);
-            c->launches++;
-            return cuda_check(c, cudaGetLastError(), "Powell step launch");
-        }
-    }
+    IdealArgs<C> a = make_step_args<C>(c);
     if constexpr (D == 3 && Codec<S>::kDev) {
         if (d.nx % 8 == 0) {  // 16-byte aligned rows: bulk-copy loads, persistent CTAs
             if (c->bulk_ctas == 0) {  // every SM filled to the kernel's occupancy
@@ -852,7 +833,7 @@ template <int D, class S, class C> vlbm_status step_t(vlbm_ctx *c, int parity)
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ideal_step_pairs<S, false>, kPairThreads, 0);
                 c->bulk_ctas = std::max(1, sms) * std::max(1, per_sm);
             }
-            const int ntiles = (int)grid.x * d.ny * d.nz;
+            const int ntiles = (d.nx + kBlockX - 1) / kBlockX * d.ny * d.nz;
             const unsigned g = (unsigned)std::min(ntiles, c->bulk_ctas);
             if (parity)
                 k_ideal_step_pairs<S, true><<<g, kPairThreads, 0, c->stream>>>(a);
@@ -862,19 +843,25 @@ template <int D, class S, class C> vlbm_status step_t(vlbm_ctx *c, int parity)
             return cuda_check(c, cudaGetLastError(), "ideal step launch");
         }
     }
-    if constexpr (Codec<S>::kDev) {
-        if (parity)
-            k_ideal_step_dev<D, S, true><<<grid, kBlockX, 0, c->stream>>>(a);
-        else
-            k_ideal_step_dev<D, S, false><<<grid, kBlockX, 0, c->stream>>>(a);
-    } else {
-        if (parity)
-            k_ideal_step<D, S, C, true><<<grid, kBlockX, 0, c->stream>>>(a);
-        else
-            k_ideal_step<D, S, C, false><<<grid, kBlockX, 0, c->stream>>>(a);
-    }
+    const StepGrid g = step_grid(d.nx, d.ny, d.nz);
+    a.by_nx = g.nx;
+    const char *what = "ideal step launch";
+    with_flags(parity != 0, g.planes, [&](auto odd, auto planes) {
+        constexpr bool O = decltype(odd)::value, P = decltype(planes)::value;
+        if constexpr (Codec<S>::kDev) {
+            k_ideal_step_dev<D, S, O, P><<<g.grid, kBlockX, 0, c->stream>>>(a);
+        } else if (c->solid) {  // homogenised solids
+            what = "homogenised step launch";
+            k_ideal_step<D, S, C, O, P, false, 8, true><<<g.grid, kBlockX, 0, c->stream>>>(a);
+        } else if (c->nlat == 9) {  // Powell model
+            what = "Powell step launch";
+            k_ideal_step<D, S, C, O, P, false, 9><<<g.grid, kBlockX, 0, c->stream>>>(a);
+        } else {
+            k_ideal_step<D, S, C, O, P><<<g.grid, kBlockX, 0, c->stream>>>(a);
+        }
+    });
     c->launches++;
-    return cuda_check(c, cudaGetLastError(), "ideal step launch");
+    return cuda_check(c, cudaGetLastError(), what);
 }
 
 template <int D, class S> vlbm_status init_t(vlbm_ctx *c, int di, const double *Q, int64_t c0, int64_t count,
@@ -1040,11 +1027,12 @@ vlbm_status ideal_step_corrected(vlbm_ctx *c, int parity, const float *dphi)
     const Domain &d = c->dom[0];
     IdealArgs<float> a = make_step_args<float>(c);
     a.dphi = dphi;
-    const dim3 grid((unsigned)((d.nx + kBlockX - 1) / kBlockX), (unsigned)d.ny, (unsigned)d.nz);
-    if (parity)
-        k_ideal_step<3, float, float, true, true><<<grid, kBlockX, 0, c->stream>>>(a);
-    else
-        k_ideal_step<3, float, float, false, true><<<grid, kBlockX, 0, c->stream>>>(a);
+    const StepGrid g = step_grid(d.nx, d.ny, d.nz);
+    a.by_nx = g.nx;
+    with_flags(parity != 0, g.planes, [&](auto odd, auto planes) {
+        k_ideal_step<3, float, float, decltype(odd)::value, decltype(planes)::value, true>
+            <<<g.grid, kBlockX, 0, c->stream>>>(a);
+    });
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "corrected step launch");
 }

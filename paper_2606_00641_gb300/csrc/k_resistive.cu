@@ -59,6 +59,7 @@ struct Args {
     float bw[3];           // wall field
     int walls_y;
     unsigned *flags;
+    FastDiv by_nx;
 };
 
 // Offsets of x + c (periodic) from x along each axis, for c = -1, 0, +1.
@@ -89,12 +90,11 @@ __device__ __forceinline__ int64_t nbr(const Offsets &o, int64_t cell, int cx, i
 
 __device__ __forceinline__ bool wall_row(int y, int ny, int walls) { return walls && (y == 0 || y == ny - 1); }
 
-template <bool ODD>
+template <bool ODD, bool PLANES>
 __global__ void __launch_bounds__(kBlockX, 5) k_res_step(const Args a)
 {
-    const int x = blockIdx.x * kBlockX + threadIdx.x;
-    if (x >= a.nx) return;
-    const int y = blockIdx.y, z = blockIdx.z;
+    int x, y, z;
+    if (!step_cell<PLANES>(a.nx, a.ny, a.by_nx, x, y, z)) return;
     const int64_t cell = x + (int64_t)a.nx * (y + (int64_t)a.ny * z);
     const Offsets o = offsets(x, y, z, a.nx, a.ny, a.nz);
     float *pop = a.pop;
@@ -541,12 +541,12 @@ ReadArgs make_read(vlbm_ctx *c, int di)
 vlbm_status resistive_step(vlbm_ctx *c, int parity)
 {
     const Domain &d = c->dom[0];
-    const Args a = make_args(c);
-    const dim3 grid((unsigned)((d.nx + kBlockX - 1) / kBlockX), (unsigned)d.ny, (unsigned)d.nz);
-    if (parity)
-        k_res_step<true><<<grid, kBlockX, 0, c->stream>>>(a);
-    else
-        k_res_step<false><<<grid, kBlockX, 0, c->stream>>>(a);
+    Args a = make_args(c);
+    const StepGrid g = step_grid(d.nx, d.ny, d.nz);
+    a.by_nx = g.nx;
+    with_flags(parity != 0, g.planes, [&](auto odd, auto planes) {
+        k_res_step<decltype(odd)::value, decltype(planes)::value><<<g.grid, kBlockX, 0, c->stream>>>(a);
+    });
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "resistive step launch");
 }

@@ -53,6 +53,77 @@ __host__ __device__ constexpr int opp_axis(int i) { return i == 0 ? 0 : ((i & 1)
 // operations it needs go through these helpers.
 #define VLBM_HD __host__ __device__
 
+// Unsigned 32-bit division by a launch constant (Granlund and Montgomery, 1994,
+// "Division by invariant integers using multiplication", their Figure 4.1).
+struct FastDiv {
+    uint32_t d, m, sh1, sh2;
+    VLBM_HD __forceinline__ uint32_t div(uint32_t n) const
+    {
+#ifdef __CUDA_ARCH__
+        const uint32_t t = __umulhi(m, n);
+#else
+        const uint32_t t = (uint32_t)(((uint64_t)m * n) >> 32);
+#endif
+        return (t + ((n - t) >> sh1)) >> sh2;
+    }
+};
+inline FastDiv fast_div(uint32_t d)
+{
+    uint32_t l = 0;
+    while (l < 32 && (uint64_t(1) << l) < d) ++l;
+    const uint32_t m = (uint32_t)(((uint64_t(1) << 32) * ((uint64_t(1) << l) - d)) / d + 1);
+    return {d, m, l < 1 ? l : 1, l < 1 ? 0 : l - 1};
+}
+
+// How a step's threads lie on the grid.  Rows: a CTA takes kBlockX cells of one x-row,
+// y and z from the block index.  Planes: a CTA takes kBlockX consecutive cells of an
+// xy-plane whatever row they are in, z from the block index, x and y by a division.
+// Rows leave threads without a cell where nx is no multiple of kBlockX (half of them at
+// nx = 64 or 130); where it is one, both give the same CTAs and rows need no division.
+struct StepGrid {
+    dim3 grid;
+    bool planes;
+    FastDiv nx;
+};
+inline StepGrid step_grid(int nx, int ny, int nz)
+{
+    const uint64_t plane = (uint64_t)nx * (uint64_t)ny, last = 0xFFFFFFFFull - kBlockX;
+    StepGrid g;
+    g.nx = fast_div((uint32_t)nx);
+    g.planes = nx % kBlockX != 0 && plane <= last && (plane + kBlockX - 1) / kBlockX <= 0x7FFFFFFFull;
+    if (g.planes) g.grid = dim3((unsigned)((plane + kBlockX - 1) / kBlockX), (unsigned)nz, 1);
+    else g.grid = dim3((unsigned)((nx + kBlockX - 1) / kBlockX), (unsigned)ny, (unsigned)nz);
+    return g;
+}
+// Calls f with the two run-time choices as compile-time ones.
+template <class F> void with_flags(bool first, bool second, F f)
+{
+    if (first) {
+        if (second) f(std::true_type{}, std::true_type{});
+        else f(std::true_type{}, std::false_type{});
+    } else {
+        if (second) f(std::false_type{}, std::true_type{});
+        else f(std::false_type{}, std::false_type{});
+    }
+}
+// This thread's cell; false where it has none.
+template <bool PLANES>
+__device__ __forceinline__ bool step_cell(int nx, int ny, const FastDiv &by_nx, int &x, int &y, int &z)
+{
+    if (PLANES) {
+        const uint32_t p = blockIdx.x * kBlockX + threadIdx.x;
+        const uint32_t r = by_nx.div(p);
+        x = (int)(p - r * by_nx.d);
+        y = (int)r;
+        z = (int)blockIdx.y;
+        return y < ny;
+    }
+    x = (int)(blockIdx.x * kBlockX + threadIdx.x);
+    y = (int)blockIdx.y;
+    z = (int)blockIdx.z;
+    return x < nx;
+}
+
 // Raise status bits in the flag word (atomically on the device).
 VLBM_HD __forceinline__ void raise_flag(unsigned *flags, unsigned bits)
 {
