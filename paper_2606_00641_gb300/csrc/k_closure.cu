@@ -8,8 +8,8 @@
 //
 // Convolutions are implicit GEMMs on the tcgen05 tensor cores (BF16 operands
 // in shared memory, FP32 accumulators in TMEM): k_conv_tc for the forward and
-// data-gradient passes (halo tiles loaded with TMA, the three z-taps stacked
-// along N), k_wgrad_tc for the weight and bias gradients (both operands read
+// data-gradient passes (marching along z over halo planes loaded with TMA, the
+// three z-taps stacked along N), k_wgrad_tc for the weight and bias gradients (both operands read
 // MN-major from the staged tiles, fixed-order partial sums).  Grids the
 // tcgen05 tiles do not divide fall back to mma.sync.m16n8k16 kernels (M = 16
 // cells per warp along an x-row, N = output channels, K = 27 taps x input
@@ -316,29 +316,30 @@ __global__ void __launch_bounds__(kTx * kTy * 2) k_conv_smem(const bf16 *__restr
 // ---------------------------------------------------------------------------
 // tcgen05 convolution (5th-generation tensor cores, accumulators in TMEM)
 // ---------------------------------------------------------------------------
-// Tile = 8 (x) x 16 (y) cells at one z = the M = 128 rows of one
-// tcgen05.mma.cta_group::1.kind::f16 (BF16 in, FP32 accumulate), N = 32
-// output channels (24-channel layers use zero weights for 24..31), K = 16 per
-// instruction.  The halo box (10 x 18 x 3 cells) is staged as channel-block
-// planes: plane cb holds channels 8cb..8cb+7 of every box cell (16 bytes per
-// cell), so 8 x-consecutive cells form one 128-byte core matrix and each tap
-// is only a start offset of the shared-memory descriptor: rows m = 8y + x,
-// 8-row groups 160 bytes apart (SBO), K-adjacent core matrices one plane
-// (Cin = 32) or one tap (Cin = 8) apart (LBO).  The weights of the layer sit
-// in shared memory in the same canonical K-major layout.  Persistent CTAs:
-// weights once, then one tile after another; one thread issues the MMAs,
-// tcgen05.commit arrives on an mbarrier (bounded wait), and each warp reads
-// its 32 TMEM lanes (= its 32 cells) with tcgen05.ld.
-constexpr int kTcX = 8, kTcY = 16, kTcZ = 4;  // tile: kTcZ z-slices of 128 cells (one M block each)
-constexpr int kTcHx = kTcX + 2, kTcHy = kTcY + 2, kTcHz = kTcZ + 2, kTcHalo = kTcHx * kTcHy * kTcHz;
-constexpr int kTcPlane = kTcHalo * 16;    // bytes per channel-block plane
-constexpr int kTcThreads = 480;           // warps 0-7 drain, 8-12 patch, 13 loads (TMA), 14 issues the MMAs
-constexpr int kTcStage = 160;             // patching threads (warps 8-12)
-constexpr int kTcBufs = 2;                // halo buffers
+// A column is 8 (x) x 16 (y) cells; one z-slice of it is the M = 128 rows of one
+// tcgen05.mma.cta_group::1.kind::f16 (BF16 in, FP32 accumulate), K = 16 per
+// instruction, 32 output channels per slice (24-channel layers use zero weights for
+// 24..31).  A CTA walks up a column plane by plane.  A halo plane (10 x 18 cells) is
+// staged as channel blocks: block cb holds channels 8cb..8cb+7 of every cell (16 bytes
+// per cell), so 8 x-consecutive cells form one 128-byte core matrix and each 2-D tap is
+// only a start offset of the shared-memory descriptor: rows m = 8y + x, 8-row groups
+// 160 bytes apart (SBO), K-adjacent core matrices one block (Cin = 32) or one tap
+// (Cin = 8) apart (LBO).  The weights of the layer sit in shared memory in the same
+// canonical K-major layout.
+constexpr int kTcX = 8, kTcY = 16, kTcZ = 4;  // column; grids of whole columns and a multiple of kTcZ slices
+constexpr int kTcHx = kTcX + 2, kTcHy = kTcY + 2;
+constexpr int kTcBlock = kTcHx * kTcHy * 16;  // bytes of one channel block of a halo plane
+constexpr int kTcRing = 12;               // halo planes in flight
+constexpr int kTcSlots = 16;              // accumulator blocks of 32 columns: all 512 TMEM columns
+constexpr int kTcDrain = 12;              // warps 0-11 drain (three groups of four)
+constexpr int kTcPatch = 4;               // warps 12-15 patch, 16 loads (TMA), 17 and 18 issue the MMAs
+constexpr int kTcIssue = kTcDrain + kTcPatch + 1;
+constexpr int kTcThreads = 32 * (kTcIssue + 2);
 constexpr int kTcN = 96;                  // MMA N: 3 z-taps x 32 output channels
-constexpr int kTcSetCols = 32 * (kTcZ + 4);  // one accumulator set: slices -2 .. kTcZ + 1
-constexpr int kTcCols = 2 * kTcSetCols;   // two sets = all 512 TMEM columns
 constexpr uint32_t kTcWaitLimit = 1u << 24;
+
+// bytes between ring entries: one plane, on the 128-byte boundary that TMA writes to
+constexpr int tc_plane_bytes(int cs) { return (cs / 8 * kTcBlock + 127) / 128 * 128; }
 
 // weight chunks of K = 16: (2-D tap, half of the 32 channels), or pairs of
 // 2-D taps of the 8 channels; each chunk is 96 rows (dz, output channel) x 16
@@ -347,7 +348,7 @@ constexpr int tc_nchunk(int cs) { return cs == 8 ? 5 : 18; }
 template <int CS>
 constexpr int tc_smem_bytes()
 {
-    return tc_nchunk(CS) * kTcN * 32 + kTcBufs * (CS / 8) * kTcPlane;
+    return tc_nchunk(CS) * kTcN * 32 + kTcRing * tc_plane_bytes(CS);
 }
 
 // Bounded wait for the given phase of an mbarrier.  Each try_wait may park
@@ -372,6 +373,22 @@ __device__ __forceinline__ bool tc_wait(uint32_t mb, uint32_t phase, volatile in
     }
     *abort = 1;
     return false;
+}
+
+// The same without parking: for a hand-over between two threads that is a few dozen
+// cycles away (a parked thread takes some hundred cycles to come back).
+__device__ __forceinline__ bool tc_spin(uint32_t mb, uint32_t phase, volatile int *abort)
+{
+    for (uint32_t it = 0; it < 256u; ++it) {
+        uint32_t done;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}\n"
+                     : "=r"(done)
+                     : "r"(mb), "r"(phase)
+                     : "memory");
+        if (done) return true;
+    }
+    return tc_wait(mb, phase, abort);
 }
 
 // Bounded wait that ignores the abort flag: on the way out of a CTA that gave up,
@@ -416,28 +433,82 @@ __device__ __forceinline__ void tc_mma(uint32_t dacc, uint64_t da, uint64_t db, 
                  ::"r"(dacc), "l"(da), "l"(db), "r"(idesc), "r"(acc));
 }
 
-// 3x3x3 convolution on the tcgen05 tensor cores.
-// Tile = 8 (x) x 16 (y) x kTcZ (z) cells; each z-slice is one M = 128 block.
-// The three z-taps are stacked along N: halo plane h (2-D tap (dx, dy),
-// K-chunk j) times [W(dz=0) | W(dz=1) | W(dz=2)] (N = 96) contributes to the
-// output slices h, h-1 and h-2 at once.  Slice s accumulates in the TMEM
-// columns 32 (kTcZ + 1 - s) of a set, so the three 32-column blocks that one
-// MMA writes are exactly those slices; the blocks of s = -2, -1, kTcZ,
-// kTcZ + 1 collect products that belong to no slice of the tile and are
-// never read.  One M128 x N96 x K16 MMA costs about as much as an N32 one,
-// so this takes 3 (kTcZ + 2) / (3 kTcZ) of the instructions per cell of
-// one-tap-per-MMA.  Every MMA accumulates: the drain clears the blocks it
-// reads (and all of them at start).
-// A operand: the halo, staged as 16-byte channel-block planes, so that a 2-D
-// tap is an address offset (K-major, no swizzle).  B operand: the weights,
-// resident in shared memory.  One persistent CTA per SM, three roles handing
-// work over through mbarriers:
-//   warp 13     loads the halo boxes into two buffers with TMA      (tma[b])
-//   warps 8-12  patch the periodic images on the boundary (cp.async) (full[b])
-//   warp 14     issues the MMAs of a tile into one of two TMEM sets  (empty[b], tfull[s])
-//   warps 0-7   drain a finished set: warp w reads TMEM lanes 32 (w % 4)
-//               of slices w / 4 and w / 4 + 2 (tanh derivative or bias,
-//               tanh, scale; BF16 or FP32 store), then clears them    (tempty[s])
+// The z-slices a CTA computes: the slices of all columns, column by column, cut into
+// equal contiguous shares; a share is walked as runs, one per column it touches.  A run
+// of len slices from z0 reads the len + 2 halo planes z0 - 1 .. z0 + len (periodic).
+struct TcWalk {
+    int64_t at, end;
+    int nz, tiles_x;
+    int x0, y0, z0, len;
+    __device__ __forceinline__ TcWalk(int64_t slices, int nz_, int tiles_x_) : nz(nz_), tiles_x(tiles_x_)
+    {
+        at = slices * blockIdx.x / gridDim.x;
+        end = slices * (blockIdx.x + 1) / gridDim.x;
+    }
+    __device__ __forceinline__ bool next()
+    {
+        if (at >= end) return false;
+        const int column = (int)(at / nz);
+        z0 = (int)(at - (int64_t)column * nz);
+        const int64_t left = end - at;
+        len = left < nz - z0 ? (int)left : nz - z0;
+        x0 = (column % tiles_x) * kTcX;
+        y0 = (column / tiles_x) * kTcY;
+        at += len;
+        return true;
+    }
+};
+
+// TMEM column of running slice n: 16 blocks of 32 columns used in turn, downwards.
+__device__ __forceinline__ uint32_t tc_slot(uint32_t n) { return (uint32_t)(kTcSlots - 1) - (n & (kTcSlots - 1)); }
+
+// The MMAs of one halo plane at hb: every 2-D tap and K-chunk times the weight rows that
+// start at descriptor w, added to the TMEM columns from d on.  Unrolled, so that each MMA
+// needs no more than two constant additions.
+template <int CS>
+__device__ __forceinline__ void tc_plane(uint32_t hb, uint32_t d, uint64_t w, uint32_t idesc)
+{
+    if (CS == 32) {  // chunk 2 t2 + kc: 2-D tap t2, channel blocks 2 kc and 2 kc + 1
+        const uint64_t da = tc_desc(hb, kTcBlock, kTcHx * 16);
+#pragma unroll
+        for (int j = 0; j < 18; ++j) {
+            const int t2 = j >> 1, kc = j & 1;
+            const uint32_t ofs = (uint32_t)(((t2 / 3) * kTcHx + t2 % 3) * 16 + kc * 2 * kTcBlock);
+            tc_mma(d, da + (ofs >> 4), w + (uint64_t)(j * (kTcN * 32 / 16)), idesc, 1u);
+        }
+    } else {         // chunk j: 2-D taps 2j and 2j + 1 of the single block
+#pragma unroll
+        for (int j = 0; j < tc_nchunk(8); ++j) {
+            const int t0 = 2 * j, t1 = 2 * j + 1;
+            const int o0 = ((t0 / 3) * kTcHx + t0 % 3) * 16;
+            const uint32_t lbo = t1 < 9 ? (uint32_t)(((t1 / 3) * kTcHx + t1 % 3) * 16 - o0) : 0u;
+            tc_mma(d, tc_desc(hb + (uint32_t)o0, lbo, kTcHx * 16), w + (uint64_t)(j * (kTcN * 32 / 16)), idesc,
+                   1u);  // tap 9: zero weights
+        }
+    }
+}
+
+// 3x3x3 convolution on the tcgen05 tensor cores, marching along z.
+// The three z-taps are stacked along N: halo plane h (2-D tap (dx, dy), K-chunk j)
+// times [W(dz=0) | W(dz=1) | W(dz=2)] (N = 96) contributes to the output slices h, h-1
+// and h-2 at once, whose accumulators lie in consecutive 32-column blocks (tc_slot;
+// where the ring of blocks wraps, two MMAs).  An M128 K16 MMA costs about 60 cycles for
+// any N up to 96, and the MMA issue binds: so each plane is read and multiplied once,
+// 18 MMAs (Cin = 32) a slice plus two planes a run.  Measured (launch list) against tiles
+// of four slices, which multiplied six planes for four slices: Cin = 32 at 128^3 130 -> 107
+// us, at 64^3 33 -> 22; Cin = 8 at 128^3 64 -> 59 us, at 64^3 18 -> 14.  With one issuing
+// thread, whose waits and descriptors cost some 800 cycles a plane, 132 us at 128^3; with
+// parked waits between the two, or the weights copied by the threads, slower at small sizes.
+// The accumulation order of a slice (planes upwards, chunks in order) is that of the tiles.
+// Every MMA accumulates: the drain clears each block it reads (all of them at start).
+// One persistent CTA per SM, roles handing work over through mbarriers:
+//   warp 16      loads halo planes into a ring with TMA                      (tma[b])
+//   warps 12-15  patch the periodic images beyond the x and y boundary, one
+//                plane each in turn (cp.async)                               (full[b])
+//   warps 17, 18 issue the MMAs of alternate planes         (turn, empty[b], tfull[p])
+//   warps 0-11   three groups take the finished slices in turn: warp w reads TMEM lanes
+//                32 (w % 4), clears them (tempty[p]), then applies the tanh derivative or
+//                bias, tanh, scale and stores BF16 or FP32
 template <int CS>
 __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restrict__ act, int nx, int ny, int nz,
                                                            const bf16 *__restrict__ wtc, int cout_real,
@@ -445,52 +516,48 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restric
                                                            const __grid_constant__ CUtensorMap halo_map)
 {
     constexpr int NCHUNK = tc_nchunk(CS);
-    constexpr int NPLANE = CS / 8;
+    constexpr int NBLOCK = CS / 8;
     constexpr int WBYTES = NCHUNK * kTcN * 32;
-    constexpr int HBYTES = NPLANE * kTcPlane;
+    constexpr int HBYTES = NBLOCK * kTcBlock;           // a plane's copy
+    constexpr uint32_t HSTEP = tc_plane_bytes(CS);
+    static_assert(WBYTES % 128 == 0, "TMA destinations lie on 128-byte boundaries");
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) uint64_t bar[3 * kTcBufs + 4];  // full[2], empty[2], tfull[2], tempty[2], tma[2]
+    __shared__ __align__(8) uint64_t bar[3 * kTcRing + 2 * kTcSlots + 3];  // full, empty, tma; tfull, tempty; turn[2]; weights
     __shared__ uint32_t tmem_base;
     __shared__ float s_bias[32], s_scale[32];
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = nx / kTcX, tiles_y = ny / kTcY, tiles_z = nz / kTcZ;
-    const int ntiles = tiles_x * tiles_y * tiles_z;
+    const int tiles_x = nx / kTcX;
     const int plane = nx * ny;
     const size_t N = (size_t)plane * nz;
-    const int n_my = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int64_t slices = (int64_t)tiles_x * (ny / kTcY) * nz;
     const uint32_t bar_s = (uint32_t)__cvta_generic_to_shared(bar);
-    auto full = [&](int b) { return bar_s + 8u * (uint32_t)b; };
-    auto empty = [&](int b) { return bar_s + 8u * (uint32_t)(kTcBufs + b); };
-    auto tfull = [&](int s2) { return bar_s + 8u * (uint32_t)(2 * kTcBufs + s2); };
-    auto tempty = [&](int s2) { return bar_s + 8u * (uint32_t)(2 * kTcBufs + 2 + s2); };
-    auto tma_bar = [&](int b) { return bar_s + 8u * (uint32_t)(2 * kTcBufs + 4 + b); };
-    auto slice_col = [](int zz) { return (uint32_t)(32 * (kTcZ + 1 - zz)); };
+    auto full = [&](uint32_t b) { return bar_s + 8u * b; };
+    auto empty = [&](uint32_t b) { return bar_s + 8u * (kTcRing + b); };
+    auto tma_bar = [&](uint32_t b) { return bar_s + 8u * (2 * kTcRing + b); };
+    auto tfull = [&](uint32_t p) { return bar_s + 8u * (3 * kTcRing + p); };
+    auto tempty = [&](uint32_t p) { return bar_s + 8u * (3 * kTcRing + kTcSlots + p); };
+    auto turn = [&](uint32_t q) { return bar_s + 8u * (3 * kTcRing + 2 * kTcSlots + q); };
+    const uint32_t wbar = turn(2);
 
-    for (int i = tid; i < WBYTES / 16; i += kTcThreads)
-        reinterpret_cast<uint4 *>(smem)[i] = __ldg(reinterpret_cast<const uint4 *>(wtc) + i);
     if (tid < 32) {  // absent bias / scale: 0 / 1, exact
         s_bias[tid] = e.bias && tid < cout_real ? e.bias[tid] : 0.f;
         s_scale[tid] = e.scale && tid < cout_real ? e.scale[tid] : 1.f;
     }
     if (warp == 0) {
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dst), "r"(kTcCols));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dst),
+                     "r"(32 * kTcSlots));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
-    if (tid == 0) {
-        s_abort = 0;
-        for (int b = 0; b < kTcBufs; ++b) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(full(b)), "r"(kTcStage));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(empty(b)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tma_bar(b)));
-        }
-        for (int s2 = 0; s2 < 2; ++s2) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(tfull(s2)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;\n" ::"r"(tempty(s2)));
-        }
+    constexpr int kBars = 3 * kTcRing + 2 * kTcSlots + 3;
+    if (tid < kBars) {  // arrivals per phase: 2 commits a finished slice, 4 warps a drained one, else 1
+        const int p = tid - 3 * kTcRing;
+        const uint32_t arrivals = p >= 0 && p < kTcSlots ? 2u : (p >= kTcSlots && p < 2 * kTcSlots ? 4u : 1u);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar_s + 8u * (uint32_t)tid), "r"(arrivals));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    if (tid == 0) s_abort = 0;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
@@ -499,172 +566,175 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restric
     const uint32_t sw_s = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t sh_s = sw_s + WBYTES;
     volatile int *abort = &s_abort;
-    uint32_t zero[32];
-#pragma unroll
-    for (int c = 0; c < 32; ++c) zero[c] = 0u;
     auto tmem_clear = [&](uint32_t taddr) {
-        asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-                     "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n"
-                     ::"r"(taddr), "r"(zero[0]), "r"(zero[1]), "r"(zero[2]), "r"(zero[3]), "r"(zero[4]),
-                       "r"(zero[5]), "r"(zero[6]), "r"(zero[7]), "r"(zero[8]), "r"(zero[9]), "r"(zero[10]),
-                       "r"(zero[11]), "r"(zero[12]), "r"(zero[13]), "r"(zero[14]), "r"(zero[15]), "r"(zero[16]),
-                       "r"(zero[17]), "r"(zero[18]), "r"(zero[19]), "r"(zero[20]), "r"(zero[21]), "r"(zero[22]),
-                       "r"(zero[23]), "r"(zero[24]), "r"(zero[25]), "r"(zero[26]), "r"(zero[27]), "r"(zero[28]),
-                       "r"(zero[29]), "r"(zero[30]), "r"(zero[31])
+        const uint32_t z = 0u;
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
+                     "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};\n" ::"r"(taddr), "r"(z)
                      : "memory");
     };
-    if (warp < 8) {  // clear the blocks this warp drains, in both sets
-        const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
-        for (int s2 = 0; s2 < 2; ++s2)
-            for (int p = 0; p < 2; ++p)
-                tmem_clear(tmem + lanes + (uint32_t)(s2 * kTcSetCols) + slice_col((warp >> 2) + 2 * p));
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+    if (warp < kTcDrain) {
+        for (int p = warp >> 2; p < kTcSlots; p += kTcDrain / 4) tmem_clear(tmem + lanes + (uint32_t)(32 * p));
         asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 
-    auto origin = [&](int i, int &x0, int &y0, int &z0) {
-        const int tile = (int)blockIdx.x + i * (int)gridDim.x;
-        x0 = (tile % tiles_x) * kTcX;
-        y0 = ((tile / tiles_x) % tiles_y) * kTcY;
-        z0 = (tile / (tiles_x * tiles_y)) * kTcZ;
-    };
-
-    if (warp == 13) {
-        // ---- halo loads: one thread issues, a tile ahead of the MMAs as far as the buffers allow,
-        // one bulk tensor copy per channel-block plane (box of 18 x 6 rows of 10 cells x 16 bytes,
-        // contiguous in the channel-blocked field); coordinates outside the grid read as zeros
+    TcWalk w(slices, nz, tiles_x);
+    bool ok = true;
+    if (warp == kTcDrain + kTcPatch) {
+        // ---- halo loads: one thread issues, as far ahead of the MMAs as the ring allows, one
+        // bulk tensor copy per plane (box of 18 rows of 10 cells x 16 bytes per channel block);
+        // cells beyond the x and y boundary read as zeros
         if (lane == 0) {
             const uint64_t map_addr = reinterpret_cast<uint64_t>(&halo_map);
-            bool ok = true;
-            int issued = 0;  // tiles whose halo copies this thread started
-            for (int i = 0; i < n_my && ok; ++i) {
-                const int b = i % kTcBufs;
-                if (i >= kTcBufs && !tc_wait(empty(b), (uint32_t)((i / kTcBufs - 1) & 1), abort)) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(wbar),
+                         "r"((uint32_t)WBYTES)
+                         : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                         ::"r"(sw_s), "l"(wtc), "r"((uint32_t)WBYTES), "r"(wbar)
+                         : "memory");
+            uint32_t i = 0;  // planes whose copies this thread started
+            while (ok && w.next())
+                for (int h = 0; h < w.len + 2; ++h, ++i) {
+                    const uint32_t b = i % kTcRing, use = i / kTcRing;
+                    if (use > 0 && !tc_wait(empty(b), (use - 1) & 1u, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    int z = w.z0 - 1 + h;
+                    z += z < 0 ? nz : (z >= nz ? -nz : 0);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(tma_bar(b)),
+                                 "r"((uint32_t)HBYTES)
+                                 : "memory");
+                    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+                                 " [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(sh_s + b * HSTEP),
+                                 "l"(map_addr), "r"(8 * (w.x0 - 1)), "r"(w.y0 - 1), "r"(z), "r"(0), "r"(tma_bar(b))
+                                 : "memory");
+                }
+            if (!ok || *abort) {
+                if (!ok) atomicOr(err, kFlagTimeout);
+                // the CTA gives up: the weights and the last copy of each ring entry land before it exits
+                tc_drain(wbar, 0u);
+                for (uint32_t j = i > (uint32_t)kTcRing ? i - kTcRing : 0u; j < i; ++j)
+                    tc_drain(tma_bar(j % kTcRing), (j / kTcRing) & 1u);
+            }
+        }
+    } else if (warp >= kTcDrain && warp < kTcDrain + kTcPatch) {
+        // ---- patching: once a plane has landed, planes of columns on the boundary get the
+        // periodic images of their edge cells with cp.async; then the plane goes to the MMA warp
+        uint32_t i = 0;
+        while (ok && w.next()) {
+            const bool edge = w.x0 == 0 || w.x0 + kTcX == nx || w.y0 == 0 || w.y0 + kTcY == ny;
+            for (int h = 0; h < w.len + 2; ++h, ++i) {
+                if ((i & (kTcPatch - 1)) != (uint32_t)(warp - kTcDrain)) continue;
+                const uint32_t b = i % kTcRing;
+                if (!__all_sync(0xffffffffu, tc_wait(tma_bar(b), (i / kTcRing) & 1u, abort))) {
                     ok = false;
                     break;
                 }
-                int x0, y0, z0;
-                origin(i, x0, y0, z0);
-                const uint32_t hb = sh_s + (uint32_t)(b * HBYTES);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(tma_bar(b)),
-                             "r"((uint32_t)HBYTES)
-                             : "memory");
-                for (int cb = 0; cb < NPLANE; ++cb)
-                    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                                 " [%0], [%1, {%2, %3, %4, %5}], [%6];\n" ::"r"(hb + (uint32_t)(cb * kTcPlane)),
-                                 "l"(map_addr), "r"(8 * (x0 - 1)), "r"(y0 - 1), "r"(z0 - 1), "r"(cb), "r"(tma_bar(b))
-                                 : "memory");
-                issued = i + 1;
-            }
-            if (!ok || *abort) {
-                if (!ok) atomicOr(err, kFlagTimeout);
-                // the CTA gives up: the last copies of each buffer land before it exits
-                for (int j = issued > kTcBufs ? issued - kTcBufs : 0; j < issued; ++j)
-                    tc_drain(tma_bar(j % kTcBufs), (uint32_t)((j / kTcBufs) & 1));
-            }
-        }
-    } else if (warp >= 8 && warp < 13) {
-        // ---- patching: once a tile's box has landed, tiles on the boundary get the periodic
-        // images of the out-of-grid halo cells with cp.async; then every patching thread
-        // hands the buffer to the MMA warp (full[b])
-        const int ptid = tid - 256;
-        bool ok = true;
-        for (int i = 0; i < n_my && ok; ++i) {
-            const int b = i % kTcBufs;
-            if (!tc_wait(tma_bar(b), (uint32_t)((i / kTcBufs) & 1), abort)) {
-                ok = false;
-                break;
-            }
-            int x0, y0, z0;
-            origin(i, x0, y0, z0);
-            if (x0 == 0 || x0 + kTcX == nx || y0 == 0 || y0 + kTcY == ny || z0 == 0 || z0 + kTcZ == nz) {
-                const uint32_t hb = sh_s + (uint32_t)(b * HBYTES);
-                for (int idx = ptid; idx < kTcHalo * NPLANE; idx += kTcStage) {
-                    const int cb = idx % NPLANE, c = idx / NPLANE;
-                    const int bx = c % kTcHx, by = (c / kTcHx) % kTcHy, bz = c / (kTcHx * kTcHy);
-                    int gx = x0 - 1 + bx, gy = y0 - 1 + by, gz = z0 - 1 + bz;
-                    if (gx >= 0 && gx < nx && gy >= 0 && gy < ny && gz >= 0 && gz < nz) continue;
-                    gx += gx < 0 ? nx : (gx >= nx ? -nx : 0);
-                    gy += gy < 0 ? ny : (gy >= ny ? -ny : 0);
-                    gz += gz < 0 ? nz : (gz >= nz ? -nz : 0);
-                    const size_t cell = (size_t)gx + (size_t)nx * gy + (size_t)plane * gz;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(hb + (uint32_t)(cb * kTcPlane + c * 16)),
-                                 "l"(act + ((size_t)cb * N + cell) * 8)
-                                 : "memory");
-                }
-                asm volatile("cp.async.commit_group;\n" ::: "memory");
-                asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-            }
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            tc_arrive(full(b));
-        }
-        if (!ok && ptid == 0) atomicOr(err, kFlagTimeout);
-    } else if (warp == 14) {
-        // ---- MMA issue (one thread)
-        if (lane == 0) {
-            const uint32_t idesc =
-                (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcN >> 3) << 17) | ((128u >> 4) << 24);
-            const uint64_t db0 = tc_desc(sw_s, 128, 256);
-            bool ok = true;
-            for (int i = 0; i < n_my && ok; ++i) {
-                const int b = i % kTcBufs, sa = i & 1;
-                if (!tc_wait(full(b), (uint32_t)((i / kTcBufs) & 1), abort)) ok = false;
-                if (ok && i >= 2 && !tc_wait(tempty(sa), (uint32_t)(((i >> 1) - 1) & 1), abort)) ok = false;
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t hb = sh_s + (uint32_t)(b * HBYTES);
-                for (int h = 0; h < kTcHz; ++h) {
-                    const uint32_t dacc = tmem + (uint32_t)(sa * kTcSetCols) + slice_col(h);
-                    const uint32_t pofs = (uint32_t)(h * kTcHy * kTcHx * 16);
-                    if (CS == 32) {  // chunk 2 t2 + kc: 2-D tap t2, channel blocks 2 kc and 2 kc + 1
-                        const uint64_t da0 = tc_desc(hb + pofs, kTcPlane, kTcHx * 16);
-                        int j = 0;
-                        for (int dy = 0; dy < 3; ++dy)
-                            for (int dx = 0; dx < 3; ++dx) {
-                                const uint32_t ofs = (uint32_t)((dy * kTcHx + dx) * 16);
-#pragma unroll
-                                for (int kc = 0; kc < 2; ++kc, ++j)
-                                    tc_mma(dacc, da0 + ((ofs + (uint32_t)(kc * 2 * kTcPlane)) >> 4),
-                                           db0 + (uint64_t)(j * (kTcN * 32 / 16)), idesc, 1u);
-                            }
-                    } else {         // chunk j: 2-D taps 2j and 2j + 1 of the single plane
-                        for (int j = 0; j < NCHUNK; ++j) {
-                            const int t0 = 2 * j, t1 = 2 * j + 1;
-                            const int o0 = ((t0 / 3) * kTcHx + t0 % 3) * 16;
-                            const uint32_t lbo = t1 < 9 ? (uint32_t)(((t1 / 3) * kTcHx + t1 % 3) * 16 - o0) : 0u;
-                            tc_mma(dacc, tc_desc(hb + pofs + (uint32_t)o0, lbo, kTcHx * 16),
-                                   db0 + (uint64_t)(j * (kTcN * 32 / 16)), idesc, 1u);  // tap 9: zero weights
+                if (edge) {
+                    const uint32_t hb = sh_s + b * HSTEP;
+                    int z = w.z0 - 1 + h;
+                    z += z < 0 ? nz : (z >= nz ? -nz : 0);
+                    constexpr int RIM = 2 * kTcHx + 2 * kTcY;  // cells on the rim of the 10 x 18 box
+                    for (int idx = lane; idx < RIM * NBLOCK; idx += 32) {
+                        const int cb = idx % NBLOCK, r = idx / NBLOCK;
+                        int bx, by;
+                        if (r < 2 * kTcHx) {
+                            by = r < kTcHx ? 0 : kTcHy - 1;
+                            bx = r < kTcHx ? r : r - kTcHx;
+                        } else {
+                            by = 1 + ((r - 2 * kTcHx) >> 1);
+                            bx = ((r - 2 * kTcHx) & 1) ? kTcHx - 1 : 0;
                         }
+                        int gx = w.x0 - 1 + bx, gy = w.y0 - 1 + by;
+                        if (gx >= 0 && gx < nx && gy >= 0 && gy < ny) continue;
+                        gx += gx < 0 ? nx : (gx >= nx ? -nx : 0);
+                        gy += gy < 0 ? ny : (gy >= ny ? -ny : 0);
+                        const size_t cell = (size_t)gx + (size_t)nx * gy + (size_t)plane * z;
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                                         hb + (uint32_t)(cb * kTcBlock + (by * kTcHx + bx) * 16)),
+                                     "l"(act + ((size_t)cb * N + cell) * 8)
+                                     : "memory");
                     }
+                    asm volatile("cp.async.commit_group;\n" ::: "memory");
+                    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
                 }
-                tc_commit(empty(b));
-                tc_commit(tfull(sa));
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc_arrive(full(b));
+            }
+        }
+        if (!ok && lane == 0) atomicOr(err, kFlagTimeout);
+    } else if (warp >= kTcIssue) {
+        // ---- MMA issue: two threads take the planes in turn, so that one waits for its
+        // plane and its accumulator and works out descriptors while the other's MMAs run
+        if (lane == 0) {
+            auto idesc = [](int ntap) {
+                return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(32 * ntap >> 3) << 17) | ((128u >> 4) << 24);
+            };
+            const uint64_t db0 = tc_desc(sw_s, 128, 256);
+            const uint32_t q = (uint32_t)(warp - kTcIssue);
+            uint32_t i = 0, n0 = 0;  // running plane; running slice of the run's first one
+            ok = tc_wait(wbar, 0u, abort);
+            while (ok && w.next()) {
+                for (int h = 0; h < w.len + 2; ++h, ++i) {
+                    if ((i & 1u) != q) continue;
+                    const uint32_t b = i % kTcRing, n = n0 + (uint32_t)h;
+                    if (!tc_wait(full(b), (i / kTcRing) & 1u, abort)) ok = false;
+                    if (ok && h < w.len && n >= (uint32_t)kTcSlots &&
+                        !tc_wait(tempty(tc_slot(n)), (n / kTcSlots - 1u) & 1u, abort))
+                        ok = false;
+                    if (!ok) break;
+                    // z-taps of this plane whose slices belong to the run, in one or two column ranges
+                    const int lo = h < w.len ? 0 : h - w.len + 1, hi = h < 2 ? h : 2;
+                    const uint32_t p0 = tc_slot(n - (uint32_t)lo);
+                    const int ntap = hi - lo + 1;
+                    const int n1 = min(ntap, kTcSlots - (int)p0);
+                    const uint32_t d1 = tmem + 32u * p0, d2 = tmem;
+                    const uint32_t id1 = idesc(n1), id2 = idesc(ntap - n1);
+                    const uint64_t w1 = db0 + (uint64_t)(64 * lo), w2 = w1 + (uint64_t)(64 * n1);  // 32 rows: 1024 B
+                    const uint32_t hb = sh_s + b * HSTEP;
+                    // planes in order: plane i follows the other thread's plane i - 1
+                    if (i > 0 && !tc_spin(turn(q), ((i - 1u) >> 1) & 1u, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    tc_plane<CS>(hb, d1, w1, id1);
+                    if (n1 < ntap) tc_plane<CS>(hb, d2, w2, id2);
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                    tc_arrive(turn(q ^ 1u));
+                    tc_commit(empty(b));
+                    // a commit covers its own thread's MMAs: slice s is complete with planes s and
+                    // s + 2 of one thread and plane s + 1 of the other
+                    if (h >= 1 && h <= w.len) tc_commit(tfull(tc_slot(n - 1u)));
+                    if (h >= 2) tc_commit(tfull(tc_slot(n - 2u)));
+                }
+                n0 += (uint32_t)w.len;
             }
             if (!ok) atomicOr(err, kFlagTimeout);
         }
-    } else if (warp < 8) {
+    } else {
         // ---- drain
-        const int q = warp & 3;
-        const int m = q * 32 + lane;  // tile row = x + 8 y
-        bool ok = true;
-        for (int i = 0; i < n_my && ok; ++i) {
-            const int sa = i & 1;
-            // tcgen05.ld is warp-collective: the whole warp takes one outcome
-            if (!__all_sync(0xffffffffu, tc_wait(tfull(sa), (uint32_t)((i >> 1) & 1), abort))) {
-                ok = false;
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            int x0, y0, z0;
-            origin(i, x0, y0, z0);
-#pragma unroll 1
-            for (int p = 0; p < 2; ++p) {
-                const int zz = (warp >> 2) + 2 * p;
+        const int m = (warp & 3) * 32 + lane;  // row = x + 8 y
+        const uint32_t group = (uint32_t)(warp >> 2);
+        uint32_t n0 = 0;
+        while (ok && w.next()) {
+            for (int s = 0; s < w.len; ++s) {
+                const uint32_t n = n0 + (uint32_t)s;
+                if (n % (kTcDrain / 4) != group) continue;
+                const uint32_t p = tc_slot(n);
+                // tcgen05.ld is warp-collective: the whole warp takes one outcome
+                if (!__all_sync(0xffffffffu, tc_wait(tfull(p), (n / kTcSlots) & 1u, abort))) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 uint32_t r[32];
-                const uint32_t taddr =
-                    tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(sa * kTcSetCols) + slice_col(zz);
+                const uint32_t taddr = tmem + lanes + 32u * p;
                 asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
                              "%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
                              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
@@ -676,8 +746,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restric
                              : "r"(taddr));
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
                 tmem_clear(taddr);
-                const size_t cell =
-                    (size_t)(x0 + (m & 7)) + (size_t)nx * (y0 + (m >> 3)) + (size_t)plane * (z0 + zz);
+                // read and cleared: hand the block back to the MMA warp
+                asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc_arrive(tempty(p));
+                const size_t cell = (size_t)(w.x0 + (m & 7)) + (size_t)nx * (w.y0 + (m >> 3)) +
+                                    (size_t)plane * (w.z0 + s);
                 float v[32];
                 if (e.deriv) {
 #pragma unroll
@@ -717,11 +792,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restric
                             *reinterpret_cast<float4 *>(dst + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
                 }
             }
-            // both blocks read and cleared: hand the set back to the MMA warp
-            asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            __syncwarp();
-            if (lane == 0) tc_arrive(tempty(sa));
+            n0 += (uint32_t)w.len;
         }
         if (!ok && lane == 0) atomicOr(err, kFlagTimeout);
     }
@@ -729,7 +800,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restric
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTcCols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(32 * kTcSlots));
     }
 }
 
@@ -1391,17 +1462,17 @@ EncodeTiledFn encode_tiled_fn()
     return fn;
 }
 
-// Halo box of k_conv_tc over a channel-blocked BF16 field with cs channels:
-// dimensions (8 nx, ny, nz, cs/8 planes) with the 8 channels of a cell
-// innermost, box (8 * 10, 18, kTcZ + 2, 1), so that one copy fills one
-// channel-block plane with rows of 160 contiguous bytes.
+// Halo plane of k_conv_tc over a channel-blocked BF16 field with cs channels:
+// dimensions (8 nx, ny, nz, cs/8 blocks) with the 8 channels of a cell innermost, box
+// (8 * 10, 18, 1, cs/8), so that one copy fills the channel blocks of one plane with
+// rows of 160 contiguous bytes.
 vlbm_status encode_halo_map(CUtensorMap *m, const bf16 *base, int cs, int nx, int ny, int nz)
 {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return fail(nullptr, VLBM_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
     const cuuint64_t dims[4] = {(cuuint64_t)8 * nx, (cuuint64_t)ny, (cuuint64_t)nz, (cuuint64_t)(cs / 8)};
     const cuuint64_t strides[3] = {(cuuint64_t)nx * 16, (cuuint64_t)nx * ny * 16, (cuuint64_t)nx * ny * nz * 16};
-    const cuuint32_t box[4] = {8 * kTcHx, kTcHy, kTcHz, 1};
+    const cuuint32_t box[4] = {8 * kTcHx, kTcHy, 1, (cuuint32_t)(cs / 8)};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(base), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -1410,17 +1481,21 @@ vlbm_status encode_halo_map(CUtensorMap *m, const bf16 *base, int cs, int nx, in
     return VLBM_OK;
 }
 
-// grids the tcgen05 kernels tile exactly
+// grids the tcgen05 kernels tile exactly (k_conv_tc itself takes any nz; grids with nz % 4 keep their kernels)
 bool conv_tc_ok(const vlbm_closure *cl) { return cl->nx % kTcX == 0 && cl->ny % kTcY == 0 && cl->nz % kTcZ == 0; }
 bool wgrad_tc_ok(const vlbm_closure *cl) { return cl->nx % 8 == 0 && cl->ny % 16 == 0 && cl->nz % kWgZ == 0; }
 
 vlbm_status conv(vlbm_closure *cl, int layer, const bf16 *in, bool transpose, const ConvEpilogue &e, cudaStream_t s)
 {
     if (conv_tc_ok(cl)) {
-        // tcgen05 / TMEM tiles of 8 x 16 x 4 cells
-        // persistent CTAs, one per SM (13 warps of up to 152 registers)
-        const int ntiles = (cl->nx / kTcX) * (cl->ny / kTcY) * (cl->nz / kTcZ);
-        const unsigned grid = (unsigned)std::min(ntiles, cl->sms);
+        // tcgen05 / TMEM columns of 8 x 16 cells: persistent CTAs, one per SM.  A CTA of few
+        // slices spends most of its time on the weights' copy and the two planes a run adds,
+        // so up to 64 CTAs each takes what there is and beyond that at least four slices.
+        // 32^3 (256 slices), 128 steps: 4.13 ms on 152 CTAs and 4.46 on 64 when alone, 2.96
+        // and 1.96 a run when three contexts share the GPU; 16^3 (32 slices): 3.63 ms on 32
+        // CTAs, 4.18 on 8.
+        const int64_t slices = (int64_t)(cl->nx / kTcX) * (cl->ny / kTcY) * cl->nz;
+        const unsigned grid = (unsigned)std::min<int64_t>({slices, cl->sms, std::max<int64_t>(64, slices / 4)});
         const int cout_real = transpose ? kCin[layer] : kCout[layer];
         const bf16 *w = transpose ? cl->wtc_bwd[layer] : cl->wtc_fwd[layer];
         const CUtensorMap *map = in == cl->x ? &cl->map_x
