@@ -730,10 +730,11 @@ __global__ void k_ideal_gather(const ReadArgs<D, S> a, const int64_t *__restrict
 
 // Domain sums of Q_k: each thread accumulates its cells in double, warps and
 // the CTA reduce with shuffles and shared memory, one partial per CTA goes to
-// the scratch array; k_finish_sums adds the partials in a fixed order.
+// the scratch array, and the last CTA adds the partials in a fixed order (domain_sums).
 template <int D, class S>
 __global__ void __launch_bounds__(kReduceThreads) k_ideal_partials(const ReadArgs<D, S> a, int64_t ncell,
-                                                                   double *__restrict__ partials)
+                                                                   double *partials, unsigned *ticket,
+                                                                   double *__restrict__ sums)
 {
     constexpr int Q = AxisSet<D>::Q;
     double acc[8];
@@ -748,22 +749,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_ideal_partials(const ReadArg
 #pragma unroll
         for (int k = 0; k < 8; ++k) acc[k] += (double)cell_moment<D, S>(a, cell, nb, k);
     }
-    write_partial(acc, partials);
-}
-
-// The partials of each field added in a fixed order: warp k takes field k, its lanes
-// every 32nd CTA's partial, then a shuffle tree.  (One CTA-wide tree after another
-// over the eight fields took 17 us for 1216 partials; this takes 5 for 118.)
-__global__ void __launch_bounds__(256) k_finish_sums(const double *__restrict__ partials, int nblocks, int nvar,
-                                                     double *__restrict__ sums)
-{
-    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
-    if (k >= nvar) return;
-    double v = 0.0;
-    for (int b = lane; b < nblocks; b += 32) v += partials[(int64_t)b * 8 + k];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) sums[k] = v;
+    domain_sums(acc, partials, ticket, sums);
 }
 
 // ---------------------------------------------------------------------------
@@ -927,11 +913,9 @@ template <int D, class S> vlbm_status sums_t(vlbm_ctx *c, int di, double *sums)
     const int64_t ncell = c->dom[di].ncell;
     const int blocks = reduce_blocks(ncell);
     k_ideal_partials<D, S><<<blocks, kReduceThreads, 0, c->stream>>>(make_read_args<D, S>(c, di), ncell,
-                                                                      c->d_partials);
+                                                                      c->d_partials, c->d_flags + 1, sums);
     c->launches++;
-    vlbm_status s = cuda_check(c, cudaGetLastError(), "ideal partial sums launch");
-    if (s != VLBM_OK) return s;
-    return finish_sums(c, blocks, 8, sums);
+    return cuda_check(c, cudaGetLastError(), "ideal sums launch");
 }
 
 template <int D, class S> vlbm_status open_fill_t(vlbm_ctx *c, int parity)
@@ -1011,13 +995,6 @@ template <int D, class S> struct OpenF {
 };
 
 }  // namespace
-
-vlbm_status finish_sums(vlbm_ctx *c, int blocks, int nvar, double *sums_dev)
-{
-    k_finish_sums<<<1, 256, 0, c->stream>>>(c->d_partials, blocks, nvar, sums_dev);
-    c->launches++;
-    return cuda_check(c, cudaGetLastError(), "finish sums launch");
-}
 
 vlbm_status ideal_step(vlbm_ctx *c, int parity) { return dispatch<StepF>(c, parity); }
 

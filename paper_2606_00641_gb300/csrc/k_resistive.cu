@@ -484,7 +484,8 @@ __global__ void k_res_gather(const ReadArgs a, const int64_t *__restrict__ cells
 
 template <bool ODD>
 __global__ void __launch_bounds__(kReduceThreads) k_res_partials(const ReadArgs a, int64_t ncell,
-                                                                 double *__restrict__ partials)
+                                                                 double *partials, unsigned *ticket,
+                                                                 double *__restrict__ sums)
 {
     double acc[7] = {0, 0, 0, 0, 0, 0, 0};
     for (int64_t cell = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; cell < ncell;
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_res_partials(const ReadArgs 
 #pragma unroll
         for (int v = 0; v < 7; ++v) acc[v] += q[v];
     }
-    write_partial(acc, partials);
+    domain_sums(acc, partials, ticket, sums);
 }
 
 Args make_args(vlbm_ctx *c)
@@ -600,12 +601,12 @@ vlbm_status resistive_sums(vlbm_ctx *c, int di, double *sums_dev)
     const ReadArgs a = make_read(c, di);
     const int64_t ncell = c->dom[di].ncell;
     const int blocks = reduce_blocks(ncell);
-    if (a.parity) k_res_partials<true><<<blocks, kReduceThreads, 0, c->stream>>>(a, ncell, c->d_partials);
-    else k_res_partials<false><<<blocks, kReduceThreads, 0, c->stream>>>(a, ncell, c->d_partials);
+    if (a.parity)
+        k_res_partials<true><<<blocks, kReduceThreads, 0, c->stream>>>(a, ncell, c->d_partials, c->d_flags + 1, sums_dev);
+    else
+        k_res_partials<false><<<blocks, kReduceThreads, 0, c->stream>>>(a, ncell, c->d_partials, c->d_flags + 1, sums_dev);
     c->launches++;
-    vlbm_status s = cuda_check(c, cudaGetLastError(), "resistive partial sums launch");
-    if (s != VLBM_OK) return s;
-    return finish_sums(c, blocks, 7, sums_dev);
+    return cuda_check(c, cudaGetLastError(), "resistive sums launch");
 }
 
 }  // namespace vlbm

@@ -15,6 +15,7 @@ using namespace vlbm;
 
 namespace {
 
+constexpr size_t kSumsOffset = 128, kStatusBytes = kSumsOffset + 64;  // status word ... domain sums
 constexpr int kGraphLen = 32;                  // steps per captured graph
 constexpr int64_t kStageCells = int64_t(1) << 22;  // cells per host-staging chunk
 thread_local std::string g_err;                // errors raised before a ctx exists
@@ -356,7 +357,7 @@ vlbm_status create_common(const vlbm_params *p, int count, vlbm_ctx **out)
     }
     if (s == VLBM_OK) s = cuda_check(c, cudaEventCreateWithFlags(&c->flag_event, cudaEventDisableTiming),
                                      "event create");
-    if (s == VLBM_OK) s = cuda_check(c, cudaMallocHost(&c->h_flags, 64), "pinned flag word");
+    if (s == VLBM_OK) s = cuda_check(c, cudaMallocHost(&c->h_flags, kStatusBytes), "pinned flag word");
     if (s == VLBM_OK) {
         c->pop_bytes = (size_t)total * c->elem;
         c->pop = dev_alloc(c, c->pop_bytes);
@@ -366,7 +367,7 @@ vlbm_status create_common(const vlbm_params *p, int count, vlbm_ctx **out)
             s = fail(c, VLBM_ERR_OOM, "device allocation failed");
         } else {
             c->d_flags = static_cast<unsigned *>(status);
-            c->d_sums = reinterpret_cast<double *>(static_cast<char *>(status) + 128);
+            c->d_sums = reinterpret_cast<double *>(static_cast<char *>(status) + kSumsOffset);
             c->d_partials = reinterpret_cast<double *>(static_cast<char *>(status) + 256);
             c->d_refscale = reinterpret_cast<double *>(static_cast<char *>(status) + 256 + partial_bytes);
             for (int k = 0; k < 8; ++k) {
@@ -710,14 +711,15 @@ vlbm_status vlbm_conservation(vlbm_ctx *c, int domain, double *sums)
     if (slab_ready(c) != VLBM_OK) return VLBM_ERR_STATE;
     vlbm_status s = c->model == VLBM_RESISTIVE ? resistive_sums(c, domain, c->d_sums)
                                                : ideal_sums(c, domain, c->d_sums);
+    // the status word and the sums lie in one block: one read-back, into pinned memory
     if (s == VLBM_OK)
-        s = cuda_check(c, cudaMemcpyAsync(sums, c->d_sums, std::min(c->nvar, 8) * sizeof(double), cudaMemcpyDeviceToHost,
-                                          c->stream),
+        s = cuda_check(c, cudaMemcpyAsync(c->h_flags, c->d_flags, kStatusBytes, cudaMemcpyDeviceToHost, c->stream),
                        "sums download");
+    if (s == VLBM_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "stream synchronise");
     if (s != VLBM_OK) return s;
-    unsigned flags = 0;
-    s = read_flags_sync(c, &flags);
-    if (s != VLBM_OK) return s;
+    c->flag_pending = false;
+    const unsigned flags = *c->h_flags;
+    std::memcpy(sums, reinterpret_cast<const char *>(c->h_flags) + kSumsOffset, std::min(c->nvar, 8) * sizeof(double));
     apply_flags(c, flags);
     return VLBM_OK;
 }

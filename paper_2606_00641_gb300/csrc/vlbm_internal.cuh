@@ -272,11 +272,18 @@ inline int reduce_blocks(int64_t ncell)
     return (int)(need < 1 ? 1 : need < kReduceBlocks ? need : kReduceBlocks);
 }
 
-// The CTA's sum of its threads' NV values into its row of eight partials (zeros beyond
-// NV): shuffles within the warps, then one thread per value over the warps.
-template <int NV> __device__ __forceinline__ void write_partial(const double (&acc)[NV], double *__restrict__ partials)
+// The CTA's sum of its threads' NV values into its row of eight partials: shuffles within
+// the warps, then one thread per value over the warps.  The CTA that finishes last adds
+// the partials of all, each value by one warp in a fixed order (lane l every 32nd CTA from
+// l on, then a shuffle tree), so the sums do not depend on which CTA that is.  `ticket`
+// counts finished CTAs and is left at zero.  (A second kernel for the partials, which
+// added the values one after another, took 17 us.)
+template <int NV>
+__device__ __forceinline__ void domain_sums(const double (&acc)[NV], double *partials, unsigned *ticket,
+                                            double *__restrict__ sums)
 {
     __shared__ double red[kReduceThreads / 32][8];
+    __shared__ int last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
@@ -286,12 +293,25 @@ template <int NV> __device__ __forceinline__ void write_partial(const double (&a
         if (lane == 0) red[warp][k] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 8) {
+    if (threadIdx.x < NV) {
         double v = 0.0;
-        if (threadIdx.x < NV)
-            for (int w = 0; w < kReduceThreads / 32; ++w) v += red[w][threadIdx.x];
+        for (int w = 0; w < kReduceThreads / 32; ++w) v += red[w][threadIdx.x];
         partials[(int64_t)blockIdx.x * 8 + threadIdx.x] = v;
+        __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (warp < NV) {
+        double v = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(partials + (int64_t)b * 8 + warp);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0) sums[warp] = v;
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // Per-domain description (host and device copies).
@@ -339,10 +359,10 @@ struct vlbm_ctx {
 
     void *pop = nullptr;                // population buffer
     size_t pop_bytes = 0;
-    unsigned *d_flags = nullptr;        // device status word
-    unsigned *h_flags = nullptr;        // pinned host mirror
+    unsigned *d_flags = nullptr;        // device status word; [1]: ticket of the domain sums
+    unsigned *h_flags = nullptr;        // pinned host mirror of the status block (256 bytes)
     double *d_partials = nullptr;       // reduction scratch [kReduceBlocks x 8]
-    double *d_sums = nullptr;           // reduction result [8]
+    double *d_sums = nullptr;           // reduction result [8], 128 bytes after d_flags
     double *d_refscale = nullptr;       // q_ref[8] then q_scale[8] of domain 0 (deviation storage, FP64)
     double h_refscale[16] = {};         // host copy (the upload's source; kept alive with the context)
     double *d_q = nullptr;              // staging for host fields (lazily sized)
@@ -461,8 +481,5 @@ vlbm_status narrow_fields(vlbm_ctx *c, const double *in, int nvar, int64_t n, in
 // launch that packs (face planes -> lo, hi messages) or unpacks (the reverse)
 HaloSlots halo_slots(const vlbm_ctx *c);
 vlbm_status halo_copy(vlbm_ctx *c, void *lo, void *hi, bool pack);
-
-// reduction of per-block partials into sums (k_ideal.cu)
-vlbm_status finish_sums(vlbm_ctx *c, int blocks, int nvar, double *sums_dev);
 
 }  // namespace vlbm
