@@ -810,12 +810,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_tc(const bf16 *__restric
 // holds 2-D tap j/2 and channels 16 (j%2) + k (32 input channels), or 2-D tap
 // 2j + k/8 and channel k%8 (8 input channels; 2-D tap 9 is zero).  The
 // transposed pack (data gradient) swaps the channel roles and mirrors the tap.
-__global__ void k_pack_tc(const float *__restrict__ W, int cout, int cin, int CS, int transpose,
-                          bf16 *__restrict__ out)
+__device__ __forceinline__ void pack_tc(const float *__restrict__ W, int cout, int cin, int CS, int transpose, int idx,
+                                        bf16 *__restrict__ out)
 {
-    const int nchunk = tc_nchunk(CS);
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nchunk * kTcN * 16) return;
     const int j = idx / (kTcN * 16), rem = idx % (kTcN * 16);
     const int g = rem / 128, kh = (rem / 64) % 2, r = (rem / 8) % 8, e8 = rem % 8;
     const int n = g * 8 + r, k = kh * 8 + e8;
@@ -846,13 +843,9 @@ __global__ void k_pack_tc(const float *__restrict__ W, int cout, int cin, int CS
 // Forward:   B[(t,c)][n] = W[n][c][t].
 // Transpose (backward-data): B[(t,c)][n] = W[c][n][26 - t]  (input c = a
 // forward output channel, output n = a forward input channel).
-__global__ void k_pack(const float *__restrict__ W, int cout, int cin, int CS, int NT, int transpose,
-                       uint2 *__restrict__ frag)
+__device__ __forceinline__ void pack_mma(const float *__restrict__ W, int cout, int cin, int CS, int NT, int transpose,
+                                         int idx, uint2 *__restrict__ frag)
 {
-    const int nchunk = CS == 8 ? 14 : 54;
-    const int total = nchunk * NT * 32;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
     const int lane = idx & 31, nt = (idx >> 5) % NT, j = (idx >> 5) / NT;
     const int g = lane >> 2, tg = lane & 3;
     const int n = nt * 8 + g;
@@ -882,6 +875,29 @@ __global__ void k_pack(const float *__restrict__ W, int cout, int cin, int CS, i
     out.x = pack_bf16(__float2bfloat16_rn(v[0]), __float2bfloat16_rn(v[1]));
     out.y = pack_bf16(__float2bfloat16_rn(v[2]), __float2bfloat16_rn(v[3]));
     frag[idx] = out;
+}
+
+// The five packs of a network in one launch (blockIdx.y = pack), in the layout of the
+// convolution kernels its grid takes; as ten launches in both layouts they took 31 us
+// after every Adam step, one takes 3.5.
+struct PackJob {
+    const float *W;
+    int cout, cin, cs, nt, transpose, count;
+    bf16 *tc;       // tcgen05 layout, or null
+    uint2 *frag;    // mma.sync layout
+};
+constexpr int kPackJobs = 5;
+struct PackJobs {
+    PackJob job[kPackJobs];
+};
+
+__global__ void __launch_bounds__(256) k_pack_all(const __grid_constant__ PackJobs jobs)
+{
+    const PackJob &p = jobs.job[blockIdx.y];
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= p.count) return;
+    if (p.tc) pack_tc(p.W, p.cout, p.cin, p.cs, p.transpose, idx, p.tc);
+    else pack_mma(p.W, p.cout, p.cin, p.cs, p.nt, p.transpose, idx, p.frag);
 }
 
 // ---------------------------------------------------------------------------
@@ -990,8 +1006,7 @@ __global__ void __launch_bounds__(256) k_bgrad_part(const bf16 *__restrict__ gz,
 // out[j] += sum over blocks b of part[b * count + j]: a CTA takes 32 outputs,
 // warp w sums the blocks b = w mod 8, then the eight sums are added in order
 // (a fixed order, so the result does not depend on scheduling)
-__global__ void __launch_bounds__(256) k_part_sum(const float *__restrict__ part, int nblk, int count,
-                                                  float *__restrict__ out)
+__device__ __forceinline__ void part_sum(const float *__restrict__ part, int nblk, int count, float *__restrict__ out)
 {
     __shared__ float red[8][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1009,6 +1024,24 @@ __global__ void __launch_bounds__(256) k_part_sum(const float *__restrict__ part
         for (int q = 0; q < 8; ++q) t += red[q][lane];
         out[j] += t;
     }
+}
+
+__global__ void __launch_bounds__(256) k_part_sum(const float *__restrict__ part, int nblk, int count,
+                                                  float *__restrict__ out)
+{
+    part_sum(part, nblk, count, out);
+}
+
+// The partials of the three layers in one launch (blockIdx.y = layer): 22 us as three, 13 as one.
+struct PartSums {
+    const float *part[3];
+    float *out[3];
+    int nblk, count[3];
+};
+__global__ void __launch_bounds__(256) k_part_sums(const __grid_constant__ PartSums p)
+{
+    const int l = blockIdx.y;
+    part_sum(p.part[l], p.nblk, p.count[l], p.out[l]);
 }
 
 // Weight gradient on the tcgen05 tensor cores:
@@ -1244,29 +1277,40 @@ __global__ void k_features(const double *__restrict__ Q, int N, const Norm n, bf
 }
 
 struct LossArgs {
-    float inv_sigma[8];
-    float coef;  // 2 / N
+    double w[8];   // 1 / sigma_k^2
+    double g[8];   // 2 / (N sigma_k^2)
+    double inv_n;
 };
 
-// r = (Q1 - Qt)/sigma, loss += sum r^2 / N, gq = 2 r / (sigma N)
+// r = (Q1 - Qt)/sigma, loss += sum r^2 / N, gq = 2 r / (sigma N).  blockIdx.y = field.
+// The FP64 pipe binds it, so an element takes three FP64 operations and two conversions
+// (the weights per field come from the host, 1/sigma^2 is applied to the field's sum) and
+// a CTA reduces by shuffles; before, each element was divided by N, multiplied three times by
+// 1/sigma or 2/N, and 1216 CTAs took a 255-addition tree each: 36 -> 24 us at 64^3.
+constexpr int kLossBlocks = 152;
+
 __global__ void __launch_bounds__(256) k_loss(const double *__restrict__ q1, const double *__restrict__ qt, int N,
                                               const LossArgs la, float *__restrict__ gq, double *__restrict__ loss)
 {
-    __shared__ double red[256];
+    __shared__ double red[8];
+    const int k = blockIdx.y;
+    const double g = la.g[k];
+    const size_t base = (size_t)k * N;
     double s = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 8 * N; i += gridDim.x * blockDim.x) {
-        const int k = i / N;
-        const double r = (q1[i] - qt[i]) * la.inv_sigma[k];
-        s += r * r;
-        gq[i] = (float)(la.coef * r * la.inv_sigma[k]);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const double d = q1[base + i] - qt[base + i];
+        s = fma(d, d, s);
+        gq[base + i] = (float)(g * d);
     }
-    red[threadIdx.x] = s;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if ((int)threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        atomicAdd(loss, t * la.w[k] * la.inv_n);
     }
-    if (threadIdx.x == 0) atomicAdd(loss, red[0] * 0.5 * la.coef);
 }
 
 // dL/dy[cell][3k+a] = out_scale_k * (gq_k(x + e_a) - gq_k(x - e_a)) / 2, zero for 24..31
@@ -1370,6 +1414,7 @@ struct vlbm_closure {
     unsigned *step_err = nullptr;            // where the running kernels report (errflag or a ctx flag)
     int sms = 1;                             // streaming multiprocessors of the device
     float *wpart = nullptr, *bpart = nullptr;  // per-CTA partial weight and bias gradients
+    size_t wpart_stride = 0;                   // floats between the three layers' partials
     bool tc_maps = false;                    // halo tensor maps below are encoded
     CUtensorMap map_x{}, map_a1{}, map_a2{}, map_gy{}, map_gz{};  // TMA halo boxes of the conv inputs
     vlbm::bf16 *x = nullptr, *a1 = nullptr, *a2 = nullptr, *gy = nullptr, *gz = nullptr;
@@ -1417,26 +1462,28 @@ void *cl_alloc(vlbm_closure *cl, size_t bytes)
     return p;
 }
 
+bool conv_tc_ok(const vlbm_closure *cl);
+
 vlbm_status pack_all(vlbm_closure *cl, cudaStream_t s)
 {
+    PackJobs jobs{};
+    int n = 0, most = 0;
+    auto add = [&](int l, int cs, int nt, int transpose, bf16 *tc, uint2 *frag) {
+        PackJob &p = jobs.job[n++];
+        p = PackJob{cl->theta + cl->off_W[l], kCout[l], kCin[l], cs, nt, transpose,
+                    tc ? tc_nchunk(cs) * kTcN * 16 : nchunk(cs) * nt * 32, tc, frag};
+        most = std::max(most, p.count);
+    };
+    const bool tc = conv_tc_ok(cl);  // which convolution kernels this grid takes
     for (int l = 0; l < 3; ++l) {
-        const int ntc = tc_nchunk(kCS[l]) * kTcN * 16;
-        k_pack_tc<<<(ntc + 255) / 256, 256, 0, s>>>(cl->theta + cl->off_W[l], kCout[l], kCin[l], kCS[l], 0,
-                                                     cl->wtc_fwd[l]);
-        if (l > 0) {
-            const int nt = tc_nchunk(32) * kTcN * 16;
-            k_pack_tc<<<(nt + 255) / 256, 256, 0, s>>>(cl->theta + cl->off_W[l], kCout[l], kCin[l], 32, 1,
-                                                        cl->wtc_bwd[l]);
-        }
-        const int total = nchunk(kCS[l]) * kNT[l] * 32;
-        k_pack<<<(total + 255) / 256, 256, 0, s>>>(cl->theta + cl->off_W[l], kCout[l], kCin[l], kCS[l], kNT[l], 0,
-                                                    cl->frag_fwd[l]);
-        if (l > 0) {  // transposed packs: input channels = forward outputs (stride 32), outputs = forward inputs
-            const int tt = nchunk(32) * 4 * 32;
-            k_pack<<<(tt + 255) / 256, 256, 0, s>>>(cl->theta + cl->off_W[l], kCout[l], kCin[l], 32, 4, 1,
-                                                     cl->frag_bwd[l]);
-        }
+        if (tc) add(l, kCS[l], 0, 0, cl->wtc_fwd[l], nullptr);
+        else add(l, kCS[l], kNT[l], 0, nullptr, cl->frag_fwd[l]);
+        if (l == 0) continue;
+        // transposed packs: input channels = forward outputs (stride 32), outputs = forward inputs
+        if (tc) add(l, 32, 0, 1, cl->wtc_bwd[l], nullptr);
+        else add(l, 32, 4, 1, nullptr, cl->frag_bwd[l]);
     }
+    k_pack_all<<<dim3((unsigned)((most + 255) / 256), (unsigned)n), 256, 0, s>>>(jobs);
     return cl_check(cudaGetLastError(), "closure weight packing");
 }
 
@@ -1605,17 +1652,21 @@ vlbm_status backward(vlbm_closure *cl, cudaStream_t s)
     const bool tc = wgrad_tc_ok(cl);
     const int ntiles = (cl->nx / 8) * (cl->ny / 16) * (cl->nz / kWgZ);
     const unsigned wg_grid = (unsigned)std::min(ntiles, cl->sms), b_grid = (unsigned)(2 * cl->sms);
+    PartSums sums{};
+    sums.nblk = (int)wg_grid;
     auto wgrad = [&](int l, const bf16 *g, const bf16 *a) {
         float *gW = cl->grad + cl->off_W[l];
         if (tc) {  // tensor cores; per-CTA partials (weights, then bias) summed in a fixed order
-            const int count = kCout[l] * kCin[l] * 27 + kCout[l];
+            float *part = cl->wpart + l * cl->wpart_stride;
             if (kCS[l] == 8)
                 k_wgrad_tc<8><<<wg_grid, kWgThreads, 2 * WgLayout<8>::BUF, s>>>(g, a, cl->nx, cl->ny, cl->nz,
-                                                                                kCout[l], cl->wpart, cl->step_err);
+                                                                                kCout[l], part, cl->step_err);
             else
                 k_wgrad_tc<32><<<wg_grid, kWgThreads, 2 * WgLayout<32>::BUF, s>>>(g, a, cl->nx, cl->ny, cl->nz,
-                                                                                  kCout[l], cl->wpart, cl->step_err);
-            k_part_sum<<<(count + 31) / 32, 256, 0, s>>>(cl->wpart, (int)wg_grid, count, gW);  // b follows W
+                                                                                  kCout[l], part, cl->step_err);
+            sums.part[l] = part;
+            sums.out[l] = gW;  // b follows W
+            sums.count[l] = kCout[l] * kCin[l] * 27 + kCout[l];
         } else {
             if (kCS[l] == 8)
                 k_wgrad<8><<<dim3(wgx, 27), kConvThreads, 0, s>>>(g, a, cl->nx, cl->ny, cl->nz, kCout[l], kCin[l], gW);
@@ -1640,6 +1691,11 @@ vlbm_status backward(vlbm_closure *cl, cudaStream_t s)
     if (st == VLBM_OK) st = conv(cl, 1, cl->gz, true, e, s);
     // layer 1
     if (st == VLBM_OK) st = wgrad(0, cl->gy, cl->x);
+    if (st == VLBM_OK && tc) {
+        const int most = std::max({sums.count[0], sums.count[1], sums.count[2]});
+        k_part_sums<<<dim3((unsigned)((most + 31) / 32), 3), 256, 0, s>>>(sums);
+        st = cl_check(cudaGetLastError(), "closure weight gradient sums");
+    }
     return st;
 }
 
@@ -1718,7 +1774,8 @@ vlbm_status vlbm_closure_create(const vlbm_closure_params *p, vlbm_closure **out
         cudaDeviceGetAttribute(&cl->sms, cudaDevAttrMultiProcessorCount, dev);
         cl->sms = std::max(cl->sms, 1);
     }
-    cl->wpart = (float *)A((size_t)cl->sms * (32 * 32 * 27 + 32) * 4);
+    cl->wpart_stride = (size_t)cl->sms * (32 * 32 * 27 + 32);
+    cl->wpart = (float *)A(3 * cl->wpart_stride * 4);
     cl->bpart = (float *)A((size_t)2 * cl->sms * 32 * 4);
     if (!ok) {
         vlbm_closure_destroy(cl);
@@ -1840,9 +1897,15 @@ vlbm_status loss_backward(vlbm_closure *cl, const double *Qt_dev, cudaStream_t s
     vlbm_status st = cl_check(cudaMemsetAsync(cl->loss, 0, sizeof(double), s), "closure loss clear");
     if (st == VLBM_OK) {
         LossArgs la{};
-        for (int k = 0; k < 8; ++k) la.inv_sigma[k] = (float)(1.0 / cl->p.sigma[k]);
-        la.coef = 2.0f / (float)cl->N;
-        k_loss<<<1216, 256, 0, s>>>(cl->q1, Qt_dev, cl->N, la, cl->gq, cl->loss);
+        for (int k = 0; k < 8; ++k) {
+            // 1 / sigma in single precision, as the features are normalised
+            const double inv = (double)(float)(1.0 / cl->p.sigma[k]);
+            la.w[k] = inv * inv;
+            la.g[k] = (double)(2.0f / (float)cl->N) * inv * inv;
+        }
+        la.inv_n = 0.5 * (double)(2.0f / (float)cl->N);
+        const unsigned blocks = (unsigned)std::min((cl->N + 255) / 256, kLossBlocks);
+        k_loss<<<dim3(blocks, 8), 256, 0, s>>>(cl->q1, Qt_dev, cl->N, la, cl->gq, cl->loss);
         k_grad_out<<<(cl->N + 255) / 256, 256, 0, s>>>(cl->gq, cl->nx, cl->ny, cl->nz, cl->col_scale, cl->gy);
         st = cl_check(cudaGetLastError(), "closure loss launch");
     }
