@@ -194,7 +194,66 @@ VLBM_HD __forceinline__ void ideal_collide_f64(C (&f)[8][AxisSet<D>::Q], const C
     }
 }
 
-// The collision of the FP32, 16-bit and batched steps: the constants from omega_k.
+// The collision of the 3-D FP32 steps, every rounding spelled out, so that the kernels
+// that advance one step and the one that advances two (k_ideal_double) give the same
+// bits: left to the compiler, which products are fused differs from kernel to kernel.
+// relax: a function from lattice to its constants.  The two directions of an axis get
+// +- omega phi / 2 last, as one rounded value (see relax_lattice).
+template <class W>
+__device__ __forceinline__ void ideal_collide_f32(float (&f)[8][7], const float gm1, const W &relax,
+                                                  const float *src0, const float *src1, unsigned *flags)
+{
+    float q[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        float s = f[k][0];
+#pragma unroll
+        for (int i = 1; i < 7; ++i) s = __fadd_rn(s, f[k][i]);
+        q[k] = s;
+    }
+    const float ir = __frcp_rn(q[0]);
+    const float m[3] = {q[1], q[2], q[3]}, B[3] = {q[5], q[6], q[7]};
+    const float u[3] = {__fmul_rn(m[0], ir), __fmul_rn(m[1], ir), __fmul_rn(m[2], ir)};
+    auto dot = [](const float (&a)[3], const float (&b)[3]) {
+        return __fmaf_rn(a[2], b[2], __fmaf_rn(a[1], b[1], __fmul_rn(a[0], b[0])));
+    };
+    const float B2 = dot(B, B), uB = dot(u, B);
+    const float p = __fmul_rn(gm1, __fmaf_rn(-0.5f, B2, __fmaf_rn(-0.5f, dot(m, u), q[4])));
+    const float pt = __fmaf_rn(0.5f, B2, p);
+    if (!(q[0] > 0.f) || !(p > 0.f)) raise_flag(flags, kFlagNonPhysical);
+    const float Ept = __fadd_rn(q[4], pt);
+    float phi[8][3];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        phi[0][ax] = m[ax];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            if (b < ax) {  // symmetric and antisymmetric
+                phi[1 + b][ax] = phi[1 + ax][b];
+                phi[5 + b][ax] = -phi[5 + ax][b];
+            } else {
+                const float t = __fmaf_rn(m[ax], u[b], -__fmul_rn(B[ax], B[b]));
+                phi[1 + b][ax] = ax == b ? __fadd_rn(t, pt) : t;
+                phi[5 + b][ax] = ax == b ? 0.f : __fmaf_rn(u[ax], B[b], -__fmul_rn(B[ax], u[b]));
+            }
+        }
+        phi[4][ax] = __fmaf_rn(Ept, u[ax], -__fmul_rn(B[ax], uB));
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const Relax<float> r = relax(k);
+        const float A0 = __fmaf_rn(r.ow0, q[k], src0[k]), A1 = __fmaf_rn(r.ow1, q[k], src1[k]);
+        f[k][0] = __fmaf_rn(r.omc, f[k][0], A0);
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            const float bv = __fmul_rn(r.hom, phi[k][ax]);
+            f[k][2 * ax + 1] = __fadd_rn(__fmaf_rn(r.omc, f[k][2 * ax + 1], A1), bv);
+            f[k][2 * ax + 2] = __fsub_rn(__fmaf_rn(r.omc, f[k][2 * ax + 2], A1), bv);
+        }
+    }
+}
+
+// The collision of the 2-D FP32, 16-bit and batched steps: the constants from omega_k.
 // The order of its roundings is part of the 16-bit forms' results, where another
 // FP32 rounding moves a stored value by a whole 16-bit step.
 template <int D, class C, bool DEV = false>

@@ -114,6 +114,8 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
     } else {
         // deviation storage collides on the stored deviations directly (ideal_cell.cuh)
         if constexpr (sizeof(C) == 8) ideal_collide_f64<D, C>(f, a.gm1, omega, a.src0, a.src1, a.flags);
+        else if constexpr (D == 3 && !Codec<S>::kDev && !CORR)
+            ideal_collide_f32(f, a.gm1, [&](int k) { return relax_of<3, float>(a.omega[k]); }, a.src0, a.src1, a.flags);
         else ideal_collide<D, C, Codec<S>::kDev>(f, a.gm1, a.omega, a.src0, a.src1, a.flags, a.ref, a.scale,
                                                  a.inv_scale, a.refscale, a.p_theta);
     }
@@ -406,6 +408,125 @@ __global__ void __launch_bounds__(kPairThreads, 6) k_ideal_step_pairs(const Idea
         }
         __syncthreads();  // buffer b consumed before it is refilled; edge elements visible
         cur = nxt;
+    }
+}
+
+// Two steps of the plain 3-D FP32 form in one pass: an even and an odd one, from parity 0
+// in one buffer to parity 0 in another, every population read once and written once for
+// both.  One step is bound by HBM (448 B a cell at the copy rate), so this is where a
+// large box gains.  A CTA takes a column of up to kDblX x kDblY cells over kDblZ planes
+// and walks up it.  Per plane:
+//   1. every thread (32 x (kDblY + 2): the column and a rim one cell wide) loads its
+//      cell's populations and collides them (step 1);
+//   2. what step 1 sends along x and y goes to the neighbours through shared memory
+//      (three plane buffers, so that one barrier a plane suffices); what it sends along z
+//      and keeps at rest stays in the thread's registers, as a thread keeps its cell's
+//      place from plane to plane;
+//   3. the plane below then has all that step 1 sent to it: its cells are collided again
+//      (step 2) and stored where the next even step reads them (slot i of x + c_i).
+// The rim's step 1 and the planes below and above the column are computed twice, by the
+// neighbouring CTAs too: 1.6 collisions for step 1 a cell at 30 x 6 x 16; re-read rim
+// lines come from L2.  Bound by the issue of 16 warps and by L1 throughput (rows of 32
+// start anywhere, two lines an access), at about two thirds of the copy rate.
+// The arithmetic is ideal_collide_f32's, so the result is that of two k_ideal_step
+// launches bit for bit.  Measured at 512^3, two steps: 17.64 -> 13.85 ms (15.2 -> 19.4
+// GLUPS); 256^3 2.24 -> 1.77; 128^3 0.288 -> 0.245; 96^3 0.128 -> 0.141 and 64^3 (in L2)
+// 0.029 -> 0.042 (not taken, see ideal_double_ok).  Slower: four rows (192 threads, 164
+// registers) 13.83 at 512^3 but 0.259 at 128^3; 14 rows, one CTA per SM, 17.0; 32 planes
+// 14.2 at 512^3; three CTAs of 96 registers 31.4 (spills); the next plane's populations
+// staged by cp.async 17.4 or more (4-byte copies); the z and rest values in shared memory 16.9.
+constexpr int kDblX = 30, kDblY = 6, kDblZ = 16;
+constexpr int kDblThreads = 32 * (kDblY + 2);
+constexpr int kDblSmem = 3 * 32 * kDblThreads * (int)sizeof(float);
+
+struct DoubleArgs {
+    const float *in;
+    float *out;
+    int nx, ny, nz;
+    int tile_x, tiles_x, tiles_y;  // columns of tile_x <= kDblX cells
+    int64_t stride;
+    float gm1;
+    float src0[8], src1[8];
+    Relax<float> relax[8];
+    unsigned *flags;
+};
+
+__global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArgs a)
+{
+    extern __shared__ float exchange[];  // [plane % 3][lattice and direction 1 .. 4][thread]
+    constexpr int NT = kDblThreads;
+    const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5;
+    const int tx = blockIdx.x % a.tiles_x, ty = blockIdx.x / a.tiles_x % a.tiles_y,
+              tz = blockIdx.x / a.tiles_x / a.tiles_y;
+    const int x0 = tx * a.tile_x, y0 = ty * kDblY, z0 = tz * kDblZ;
+    const int xe = min(x0 + a.tile_x, a.nx), ye = min(y0 + kDblY, a.ny), ze = min(z0 + kDblZ, a.nz);
+    int x = x0 - 1 + lx, y = y0 - 1 + ly;
+    const bool first = x <= xe && y <= ye;                            // takes part in step 1
+    const bool second = lx >= 1 && ly >= 1 && x < xe && y < ye;       // and in step 2
+    x += x < 0 ? a.nx : (x >= a.nx ? -a.nx : 0);
+    y += y < 0 ? a.ny : (y >= a.ny ? -a.ny : 0);
+    const uint32_t row = (uint32_t)a.nx, plane = row * (uint32_t)a.ny;  // cells fit 32 bits (ideal_double_ok)
+    const uint32_t at = (uint32_t)x + row * (uint32_t)y;
+    const uint32_t xm = x > 0 ? at - 1 : at + row - 1, xp = x + 1 < a.nx ? at + 1 : at + 1 - row;
+    const uint32_t ym = y > 0 ? at - row : at + plane - row, yp = y + 1 < a.ny ? at + row : at + row - plane;
+    auto relax = [&](int k) { return a.relax[k]; };
+    float rest[8], up1[8], up2[8];  // step 1: at rest on the plane below; sent up from it and from the one below that
+#pragma unroll
+    for (int k = 0; k < 8; ++k) rest[k] = up1[k] = up2[k] = 0.f;
+    int buf = 0;
+    for (int z = z0 - 1; z <= ze; ++z) {
+        float f[8][7];
+        float *mine = exchange + buf * 32 * NT + tid;
+        const float *below = exchange + (buf == 0 ? 2 : buf - 1) * 32 * NT + tid;
+        buf = buf == 2 ? 0 : buf + 1;
+        if (first) {
+            const uint32_t zc = (uint32_t)(z < 0 ? z + a.nz : (z >= a.nz ? z - a.nz : z));
+            const float *p = a.in + (at + plane * zc);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int i = 0; i < 7; ++i) f[k][i] = p[(int64_t)(k * 7 + i) * a.stride];
+            ideal_collide_f32(f, a.gm1, relax, a.src0, a.src1, a.flags);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int i = 1; i < 5; ++i) mine[(k * 4 + i - 1) * NT] = f[k][i];
+            // what step 2 of the plane below gets along z and from its own cell; f[k][6] is
+            // already what this plane sends down
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float r = f[k][0], u = f[k][5];
+                f[k][0] = rest[k];
+                f[k][5] = up2[k];
+                rest[k] = r;
+                up2[k] = up1[k];
+                up1[k] = u;
+            }
+        }
+        // the plane's exchange buffer is written; the one read below was, before the last
+        // barrier, and is written again after the next one
+        __syncthreads();
+        if (z > z0 && second) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                f[k][1] = below[(k * 4 + 0) * NT - 1];
+                f[k][2] = below[(k * 4 + 1) * NT + 1];
+                f[k][3] = below[(k * 4 + 2) * NT - 32];
+                f[k][4] = below[(k * 4 + 3) * NT + 32];
+            }
+            ideal_collide_f32(f, a.gm1, relax, a.src0, a.src1, a.flags);
+            const int zo = z - 1;
+            const uint32_t pz = plane * (uint32_t)zo;
+            const uint32_t pp = plane * (uint32_t)(zo + 1 < a.nz ? zo + 1 : 0);
+            const uint32_t pm = plane * (uint32_t)(zo > 0 ? zo - 1 : a.nz - 1);
+            const uint32_t to[7] = {at + pz, xp + pz, xm + pz, yp + pz, ym + pz, at + pp, at + pm};
+#pragma unroll
+            for (int i = 0; i < 7; ++i) {
+                float *o = a.out + to[i];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) o[(int64_t)(k * 7 + i) * a.stride] = f[k][i];
+            }
+        }
     }
 }
 
@@ -997,6 +1118,74 @@ template <int D, class S> struct OpenF {
 }  // namespace
 
 vlbm_status ideal_step(vlbm_ctx *c, int parity) { return dispatch<StepF>(c, parity); }
+
+// Columns of the two-step pass over a box.
+static void double_tiles(const Domain &d, int &tile_x, int &tiles_x, int &tiles_y, int &tiles_z)
+{
+    tiles_x = (d.nx + kDblX - 1) / kDblX;
+    tile_x = (d.nx + tiles_x - 1) / tiles_x;
+    tiles_y = (d.ny + kDblY - 1) / kDblY;
+    tiles_z = (d.nz + kDblZ - 1) / kDblZ;
+}
+
+// Where the two-step pass is taken: plain 3-D FP32 boxes whose populations exceed L2
+// (below, a step is not bound by HBM) and whose columns fill the CTA slots well: of the
+// cells that all waves of CTAs could produce, rims and end planes included, at least 0.7
+// are wanted cells.  The gain is proportional to that share: 1.27 at 512^3 (0.84), 1.17 at
+// 128^3 (0.71), 0.91 at 96^3 (0.45).
+bool ideal_double_ok(vlbm_ctx *c)
+{
+    if (c->batched || c->model != VLBM_IDEAL || c->nlat != 8 || c->dim != 3 || c->storage != VLBM_F32 || c->slab ||
+        c->closure || c->solid || any_open_face(c))
+        return false;
+    const Domain &d = c->dom[0];
+    if (c->pop_bytes < (size_t(128) << 20) || d.ncell > (int64_t(1) << 30)) return false;
+    if (c->double_slots == 0) {
+        int dev = 0, sms = 0, per_sm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (cudaFuncSetAttribute(k_ideal_double, cudaFuncAttributeMaxDynamicSharedMemorySize, kDblSmem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ideal_double, kDblThreads, kDblSmem) !=
+                cudaSuccess) {
+            cudaGetLastError();
+            per_sm = 0;
+        }
+        c->double_slots = per_sm > 0 ? sms * per_sm : -1;
+    }
+    if (c->double_slots < 0) return false;
+    int tile_x, tiles_x, tiles_y, tiles_z;
+    double_tiles(d, tile_x, tiles_x, tiles_y, tiles_z);
+    const int64_t ctas = (int64_t)tiles_x * tiles_y * tiles_z;
+    const int64_t waves = (ctas + c->double_slots - 1) / c->double_slots;
+    const double could = (double)waves * c->double_slots * (kDblX * kDblY) * (kDblZ + 2);
+    return ctas <= 0x7FFFFFFF && (double)d.ncell >= 0.7 * could;
+}
+
+// One even and one odd step of every cell, `in` (parity 0) to `out` (parity 0).
+vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out)
+{
+    const Domain &d = c->dom[0];
+    const IdealArgs<float> s = make_step_args<float>(c);
+    DoubleArgs a{};
+    a.in = static_cast<const float *>(in);
+    a.out = static_cast<float *>(out);
+    a.nx = d.nx;
+    a.ny = d.ny;
+    a.nz = d.nz;
+    a.stride = d.stride;
+    a.gm1 = s.gm1;
+    for (int k = 0; k < 8; ++k) {
+        a.src0[k] = s.src0[k];
+        a.src1[k] = s.src1[k];
+        a.relax[k] = relax_of<3, float>(s.omega[k]);
+    }
+    a.flags = c->d_flags;
+    int tiles_z;
+    double_tiles(d, a.tile_x, a.tiles_x, a.tiles_y, tiles_z);
+    k_ideal_double<<<(unsigned)(a.tiles_x * a.tiles_y * tiles_z), kDblThreads, kDblSmem, c->stream>>>(a);
+    c->launches++;
+    return cuda_check(c, cudaGetLastError(), "two-step launch");
+}
 
 vlbm_status ideal_step_corrected(vlbm_ctx *c, int parity, const float *dphi)
 {

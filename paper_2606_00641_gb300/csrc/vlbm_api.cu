@@ -223,6 +223,45 @@ vlbm_status launch_step(vlbm_ctx *c, int parity)
     return s;
 }
 
+// The second population buffer of the two-step pass, once per context and only where
+// memory is plentiful: a box of at most a sixth of the device's memory, with at least
+// twice that much free beside it.  Without it (or while the stream is being captured by
+// the caller, when nothing may be allocated) every step is a launch of its own.
+void ensure_second_buffer(vlbm_ctx *c)
+{
+    if (c->pop2 || c->pop2_tried || !ideal_double_ok(c)) return;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return;
+    }
+    c->pop2_tried = true;
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (c->pop_bytes > total / 6 || c->pop_bytes > avail / 3) return;
+    c->pop2 = dev_alloc(c, c->pop_bytes);
+}
+
+// Launches the next of `left` steps from `parity`: four at once by two two-step passes,
+// out to the second buffer and back, where that pass applies (the populations are in the
+// first buffer whenever a call returns); else one.  Returns how many in *taken.  The
+// caller allows pairs where its run of steps begins at an even step count; a run that
+// begins at an odd one keeps its launch per step, as vlbm_launch_count has reported it.
+vlbm_status launch_next(vlbm_ctx *c, bool pairs, int parity, int left, int *taken)
+{
+    if (pairs && c->pop2 && parity == 0 && left >= 4 && ideal_double_ok(c)) {
+        *taken = 4;
+        vlbm_status s = ideal_double(c, c->pop, c->pop2);
+        if (s == VLBM_OK) s = ideal_double(c, c->pop2, c->pop);
+        return s;
+    }
+    *taken = 1;
+    return launch_step(c, parity);
+}
+
 vlbm_status init_range(vlbm_ctx *c, int d, const double *Q, int64_t c0, int64_t n, int64_t qs)
 {
     if (c->model == VLBM_RESISTIVE) return resistive_init_range(c, d, Q, c0, n, qs);
@@ -287,7 +326,8 @@ cudaGraphExec_t get_graph(vlbm_ctx *c, int parity, int len, int64_t *launches)
     }
     const int64_t before = c->launches;
     bool ok = true;
-    for (int s = 0; s < len && ok; ++s) ok = launch_step(c, (parity + s) & 1) == VLBM_OK;
+    for (int s = 0, taken = 0; s < len && ok; s += taken)
+        ok = launch_next(c, parity == 0, (parity + s) & 1, len - s, &taken) == VLBM_OK;
     const int64_t captured = c->launches - before;
     c->launches = before;
     cudaGraph_t g = nullptr;
@@ -578,6 +618,8 @@ vlbm_status vlbm_step(vlbm_ctx *c, int n)
             return fail(c, VLBM_ERR_ARG, "one face of an axis is open and the other periodic");
     const bool graphs = c->stream != nullptr && c->stream != cudaStreamLegacy &&
                         c->stream != cudaStreamPerThread;
+    const bool pairs = (c->step & 1) == 0;
+    if (pairs && n >= 4) ensure_second_buffer(c);
     int left = n;
     while (left > 0) {
         if (graphs && left >= kGraphLen) {
@@ -592,10 +634,11 @@ vlbm_status vlbm_step(vlbm_ctx *c, int n)
                 continue;
             }
         }
-        vlbm_status s = launch_step(c, (int)(c->step & 1));
+        int taken = 0;
+        vlbm_status s = launch_next(c, pairs, (int)(c->step & 1), left, &taken);
         if (s != VLBM_OK) return s;
-        c->step += 1;
-        left -= 1;
+        c->step += taken;
+        left -= taken;
         if (c->slab) c->halo_pending = true;
     }
     schedule_check(c, n);

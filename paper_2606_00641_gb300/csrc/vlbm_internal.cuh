@@ -374,6 +374,9 @@ struct vlbm_ctx {
     bool own_stream = false;
     cudaStream_t copy_stream = nullptr;  // host-field staging copies (overlap the chunk kernels)
     int bulk_ctas = 0;                   // persistent grid of the bulk-load step (0: not sized yet)
+    int double_slots = 0;                // CTAs of the two-step pass that the device holds (0: not asked yet)
+    void *pop2 = nullptr;                // the two-step pass's other buffer (scratch between its two launches)
+    bool pop2_tried = false;
     cudaEvent_t ev_copy[2]{}, ev_kern[2]{};  // per staging buffer: last copy / last kernel done
     cudaEvent_t flag_event = nullptr;
     bool flag_pending = false;
@@ -434,6 +437,8 @@ vlbm_status ideal_init(vlbm_ctx *c, int d, const double *Q_dev);
 vlbm_status ideal_init_range(vlbm_ctx *c, int d, const double *Q, int64_t c0, int64_t n, int64_t qstride);
 vlbm_status ideal_moments_range(vlbm_ctx *c, int d, double *out, int64_t c0, int64_t n, int64_t ostride);
 vlbm_status ideal_step(vlbm_ctx *c, int parity);
+bool ideal_double_ok(vlbm_ctx *c);
+vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out);
 vlbm_status ideal_moments(vlbm_ctx *c, int d, double *Q_dev);
 vlbm_status ideal_gather(vlbm_ctx *c, int d, const int64_t *cells_dev, int n, double *out_dev);
 vlbm_status ideal_sums(vlbm_ctx *c, int d, double *sums_dev);

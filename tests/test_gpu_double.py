@@ -1,0 +1,92 @@
+"""The two-step pass of large plain 3-D FP32 boxes: bit for bit the single steps.
+
+A run advanced in one call (pairs of steps in one pass) equals the same run advanced
+one step per call (a launch per step) in every population, at even and odd step
+counts, from an odd step count, with sources, on boxes whose sides divide neither the
+pass's columns (30 x 6) nor its height (16), and through captured graphs; and the
+oracle's result on light-cone boxes at the repository's FP32 tolerance."""
+import numpy as np
+import pytest
+
+from paper_2606_00641_gb300 import fields
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def V():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2606_00641_gb300 import vlbm
+    vlbm.load()
+    return vlbm
+
+
+def populations(V, ctx, shape, seed):
+    n = int(np.prod(shape))
+    cells = np.unique(np.concatenate([np.random.default_rng(seed).integers(0, n, 200000), np.arange(3000),
+                                      np.arange(n - 3000, n)]))
+    return ctx.populations(cells)
+
+
+@pytest.mark.parametrize("shape,calls", [((128, 128, 128), (4,)), ((128, 128, 128), (1, 7, 8, 6)),
+                                         ((161, 127, 178), (9, 6)), ((200, 149, 149), (40, 3)),
+                                         ((111, 203, 239), (70,))])
+def test_equals_single_steps(V, shape, calls):
+    import torch
+    f0 = fields.ideal_fields(shape, 21, mach=0.5, beta=1.0, cfl=0.2, device=torch.device("cuda"))
+    tau = np.array([0.51, 0.6, 0.55, 0.7, 0.52, 0.8, 0.65, 0.9])
+    src = np.array([1e-7, -2e-7, 3e-7, 0.0, 1e-8, 2e-8, -1e-8, 0.0])
+    p = V.make_params(shape=shape, storage="f32", gamma=f0.gamma, tau=tau, source=src)
+    got = []
+    for one in (False, True):
+        with V.Context(p) as ctx:
+            assert V.vlbm_init_fields_device(ctx.ptr, 0, f0.Q.data_ptr()) == V.VLBM_OK
+            before = ctx.launches
+            for n in calls:
+                for _ in range(n if one else 1):
+                    assert ctx.step(1 if one else n) == V.VLBM_OK
+            assert ctx.step_count == sum(calls)
+            passes = ctx.launches - before
+            assert ctx.sync() == V.VLBM_OK
+            got.append(populations(V, ctx, shape, 22))
+            # a launch per step, or two per four steps in calls that begin at an even step count
+            want, at = 0, 0
+            for n in calls:
+                want += n // 4 * 2 + n % 4 if at % 2 == 0 else n
+                at += n
+            assert passes == (sum(calls) if one else want)
+    assert np.array_equal(got[0], got[1])
+
+
+def test_refused_second_buffer_takes_single_steps(V):
+    """An allocator that has no second buffer to give: every step its own launch, same state."""
+    import torch
+    shape = (128, 128, 128)
+    f0 = fields.ideal_fields(shape, 23, mach=0.5, beta=1.0, cfl=0.2, device=torch.device("cuda"))
+    base = V.TorchHooks()
+    big = 56 * int(np.prod(shape)) * 4
+    seen = []
+
+    def once(nbytes, stream, user):
+        if nbytes >= big:
+            seen.append(nbytes)
+            if len(seen) > 1:
+                return None
+        return base.alloc(nbytes, stream, user)
+
+    base_alloc = V.ALLOC_FN(once)
+
+    class Hooks:
+        alloc, dealloc = base_alloc, base.dealloc
+
+    out = []
+    for hooks in (Hooks, None):
+        with V.Context(V.make_params(shape=shape, storage="f32", gamma=f0.gamma, tau=0.6, hooks=hooks)) as ctx:
+            V.vlbm_init_fields_device(ctx.ptr, 0, f0.Q.data_ptr())
+            n0 = ctx.launches
+            assert ctx.step(8) == V.VLBM_OK and ctx.sync() == V.VLBM_OK
+            out.append((ctx.launches - n0, populations(V, ctx, shape, 24)))
+    assert len(seen) == 2 and out[0][0] == 8 and out[1][0] == 4
+    assert np.array_equal(out[0][1], out[1][1])
