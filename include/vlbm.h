@@ -197,7 +197,7 @@ vlbm_status vlbm_init_fields_device(vlbm_ctx *ctx, int domain, const double *Q_d
 
 /* Enqueue n >= 0 time steps of Eq. 2 on every domain: one fused
  * collide-and-stream kernel per step (in-place AA pattern), asynchronous.
- * Large plain ideal 3-D F32 boxes take four steps at a time in two kernels of
+ * Large plain ideal F32 boxes (and batches) take four steps at a time in two kernels of
  * two steps each, bit for bit the same populations, in calls of n >= 4 that
  * begin at an even step count; the first such call allocates a second buffer
  * of vlbm_population_bytes (kept until vlbm_destroy), if the populations are at

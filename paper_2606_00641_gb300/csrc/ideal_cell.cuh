@@ -194,21 +194,22 @@ VLBM_HD __forceinline__ void ideal_collide_f64(C (&f)[8][AxisSet<D>::Q], const C
     }
 }
 
-// The collision of the 3-D FP32 steps, every rounding spelled out, so that the kernels
-// that advance one step and the one that advances two (k_ideal_double) give the same
+// The collision of the FP32 steps, every rounding spelled out, so that the kernels that
+// advance one step and those that advance two (k_ideal_double, k_double_2d) give the same
 // bits: left to the compiler, which products are fused differs from kernel to kernel.
-// relax: a function from lattice to its constants.  The two directions of an axis get
+// relax: a function from lattice to its constants and source terms.  The two directions of an axis get
 // +- omega phi / 2 last, as one rounded value (see relax_lattice).
-template <class W>
-__device__ __forceinline__ void ideal_collide_f32(float (&f)[8][7], const float gm1, const W &relax,
-                                                  const float *src0, const float *src1, unsigned *flags)
+template <int D, class W>
+__device__ __forceinline__ void ideal_collide_f32(float (&f)[8][AxisSet<D>::Q], const float gm1, const W &relax,
+                                                  unsigned *flags)
 {
+    constexpr int Q = AxisSet<D>::Q;
     float q[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         float s = f[k][0];
 #pragma unroll
-        for (int i = 1; i < 7; ++i) s = __fadd_rn(s, f[k][i]);
+        for (int i = 1; i < Q; ++i) s = __fadd_rn(s, f[k][i]);
         q[k] = s;
     }
     const float ir = __frcp_rn(q[0]);
@@ -222,9 +223,9 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[8][7], const float 
     const float pt = __fmaf_rn(0.5f, B2, p);
     if (!(q[0] > 0.f) || !(p > 0.f)) raise_flag(flags, kFlagNonPhysical);
     const float Ept = __fadd_rn(q[4], pt);
-    float phi[8][3];
+    float phi[8][D];
 #pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
+    for (int ax = 0; ax < D; ++ax) {
         phi[0][ax] = m[ax];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
@@ -241,11 +242,11 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[8][7], const float 
     }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const Relax<float> r = relax(k);
-        const float A0 = __fmaf_rn(r.ow0, q[k], src0[k]), A1 = __fmaf_rn(r.ow1, q[k], src1[k]);
+        const RelaxSource r = relax(k);
+        const float A0 = __fmaf_rn(r.ow0, q[k], r.src0), A1 = __fmaf_rn(r.ow1, q[k], r.src1);
         f[k][0] = __fmaf_rn(r.omc, f[k][0], A0);
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
+        for (int ax = 0; ax < D; ++ax) {
             const float bv = __fmul_rn(r.hom, phi[k][ax]);
             f[k][2 * ax + 1] = __fadd_rn(__fmaf_rn(r.omc, f[k][2 * ax + 1], A1), bv);
             f[k][2 * ax + 2] = __fsub_rn(__fmaf_rn(r.omc, f[k][2 * ax + 2], A1), bv);
@@ -253,7 +254,7 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[8][7], const float 
     }
 }
 
-// The collision of the 2-D FP32, 16-bit and batched steps: the constants from omega_k.
+// The collision of the 16-bit and corrected steps: the constants from omega_k.
 // The order of its roundings is part of the 16-bit forms' results, where another
 // FP32 rounding moves a stored value by a whole 16-bit step.
 template <int D, class C, bool DEV = false>

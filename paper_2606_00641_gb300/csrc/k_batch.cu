@@ -79,7 +79,8 @@ __global__ void __launch_bounds__(TX, 640 / TX) k_batch_step(const int2 *__restr
                     const int64_t at = ODD ? nb[opp_axis(i)] : cell;
                     f[k][i] = base[(int64_t)(k * Q + j) * stride + at];
                 }
-            ideal_collide<D, float>(f, gm1, omega, src0, src1, flags);
+            ideal_collide_f32<D>(
+                f, gm1, [&](int k) { return relax_source<D>(omega[k], src0[k], src1[k]); }, flags);
             // the stride is per-domain (not a kernel parameter): recompute the
             // store addresses rather than hold 40 offsets across the collision
             const int64_t sst = opaque(stride);

@@ -114,8 +114,9 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
     } else {
         // deviation storage collides on the stored deviations directly (ideal_cell.cuh)
         if constexpr (sizeof(C) == 8) ideal_collide_f64<D, C>(f, a.gm1, omega, a.src0, a.src1, a.flags);
-        else if constexpr (D == 3 && !Codec<S>::kDev && !CORR)
-            ideal_collide_f32(f, a.gm1, [&](int k) { return relax_of<3, float>(a.omega[k]); }, a.src0, a.src1, a.flags);
+        else if constexpr (!Codec<S>::kDev && !CORR)
+            ideal_collide_f32<D>(
+                f, a.gm1, [&](int k) { return relax_source<D>(a.omega[k], a.src0[k], a.src1[k]); }, a.flags);
         else ideal_collide<D, C, Codec<S>::kDev>(f, a.gm1, a.omega, a.src0, a.src1, a.flags, a.ref, a.scale,
                                                  a.inv_scale, a.refscale, a.p_theta);
     }
@@ -446,8 +447,7 @@ struct DoubleArgs {
     int tile_x, tiles_x, tiles_y;  // columns of tile_x <= kDblX cells
     int64_t stride;
     float gm1;
-    float src0[8], src1[8];
-    Relax<float> relax[8];
+    RelaxSource relax[8];
     unsigned *flags;
 };
 
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArg
             for (int k = 0; k < 8; ++k)
 #pragma unroll
                 for (int i = 0; i < 7; ++i) f[k][i] = p[(int64_t)(k * 7 + i) * a.stride];
-            ideal_collide_f32(f, a.gm1, relax, a.src0, a.src1, a.flags);
+            ideal_collide_f32<3>(f, a.gm1, relax, a.flags);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
 #pragma unroll
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArg
                 f[k][3] = below[(k * 4 + 2) * NT - 32];
                 f[k][4] = below[(k * 4 + 3) * NT + 32];
             }
-            ideal_collide_f32(f, a.gm1, relax, a.src0, a.src1, a.flags);
+            ideal_collide_f32<3>(f, a.gm1, relax, a.flags);
             const int zo = z - 1;
             const uint32_t pz = plane * (uint32_t)zo;
             const uint32_t pp = plane * (uint32_t)(zo + 1 < a.nz ? zo + 1 : 0);
@@ -1174,11 +1174,7 @@ vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out)
     a.nz = d.nz;
     a.stride = d.stride;
     a.gm1 = s.gm1;
-    for (int k = 0; k < 8; ++k) {
-        a.src0[k] = s.src0[k];
-        a.src1[k] = s.src1[k];
-        a.relax[k] = relax_of<3, float>(s.omega[k]);
-    }
+    for (int k = 0; k < 8; ++k) a.relax[k] = relax_source<3>(s.omega[k], s.src0[k], s.src1[k]);
     a.flags = c->d_flags;
     int tiles_z;
     double_tiles(d, a.tile_x, a.tiles_x, a.tiles_y, tiles_z);

@@ -223,13 +223,15 @@ vlbm_status launch_step(vlbm_ctx *c, int parity)
     return s;
 }
 
-// The second population buffer of the two-step pass, once per context and only where
-// memory is plentiful: a box of at most a sixth of the device's memory, with at least
+// The second population buffer of the two-step passes, once per context and only where
+// memory is plentiful: populations of at most a sixth of the device's memory, with at least
 // twice that much free beside it.  Without it (or while the stream is being captured by
 // the caller, when nothing may be allocated) every step is a launch of its own.
+bool double_ok(vlbm_ctx *c) { return c->dim == 3 ? ideal_double_ok(c) : double_2d_ok(c); }
+
 void ensure_second_buffer(vlbm_ctx *c)
 {
-    if (c->pop2 || c->pop2_tried || !ideal_double_ok(c)) return;
+    if (c->pop2 || c->pop2_tried || !double_ok(c)) return;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
@@ -242,6 +244,7 @@ void ensure_second_buffer(vlbm_ctx *c)
         return;
     }
     if (c->pop_bytes > total / 6 || c->pop_bytes > avail / 3) return;
+    if (c->dim == 2 && double_2d_prepare(c) != VLBM_OK) return;
     c->pop2 = dev_alloc(c, c->pop_bytes);
 }
 
@@ -252,10 +255,11 @@ void ensure_second_buffer(vlbm_ctx *c)
 // begins at an odd one keeps its launch per step, as vlbm_launch_count has reported it.
 vlbm_status launch_next(vlbm_ctx *c, bool pairs, int parity, int left, int *taken)
 {
-    if (pairs && c->pop2 && parity == 0 && left >= 4 && ideal_double_ok(c)) {
+    if (pairs && c->pop2 && parity == 0 && left >= 4 && double_ok(c)) {
         *taken = 4;
-        vlbm_status s = ideal_double(c, c->pop, c->pop2);
-        if (s == VLBM_OK) s = ideal_double(c, c->pop2, c->pop);
+        auto pass = c->dim == 3 ? ideal_double : double_2d;
+        vlbm_status s = pass(c, c->pop, c->pop2);
+        if (s == VLBM_OK) s = pass(c, c->pop2, c->pop);
         return s;
     }
     *taken = 1;

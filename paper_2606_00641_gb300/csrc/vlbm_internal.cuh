@@ -178,6 +178,11 @@ template <class C> struct Relax {
     C omc, ow0, ow1, hom;
 };
 
+// With the source terms w_0 S_k and w_moving S_k.
+struct RelaxSource {
+    float omc, ow0, ow1, hom, src0, src1;
+};
+
 // The same for N lattices, worked out once on the host and passed as kernel
 // parameters, so that an FP64 collision reads them as constant operands.  Formed
 // from omega in every thread instead they were five operations per lattice and
@@ -196,6 +201,12 @@ template <int D, class C> VLBM_HD __forceinline__ Relax<C> relax_of(C om)
     relax_weights<D, C>(om, r.ow0, r.ow1);
     r.hom = C(0.5) * om;
     return r;
+}
+
+template <int D> VLBM_HD __forceinline__ RelaxSource relax_source(float om, float src0, float src1)
+{
+    const Relax<float> r = relax_of<D, float>(om);
+    return {r.omc, r.ow0, r.ow1, r.hom, src0, src1};
 }
 
 // The constants of lattice k from the table, or worked out from omega[k].
@@ -374,7 +385,10 @@ struct vlbm_ctx {
     bool own_stream = false;
     cudaStream_t copy_stream = nullptr;  // host-field staging copies (overlap the chunk kernels)
     int bulk_ctas = 0;                   // persistent grid of the bulk-load step (0: not sized yet)
-    int double_slots = 0;                // CTAs of the two-step pass that the device holds (0: not asked yet)
+    int double_slots = 0;                // CTAs (2-D: strips) of the two-step pass that the device holds
+                                         // (0: not asked yet, -1: the pass is not taken)
+    void *double_doms = nullptr, *double_tiles = nullptr;  // 2-D: its constants and strip table
+    int double_ntiles = 0;
     void *pop2 = nullptr;                // the two-step pass's other buffer (scratch between its two launches)
     bool pop2_tried = false;
     cudaEvent_t ev_copy[2]{}, ev_kern[2]{};  // per staging buffer: last copy / last kernel done
@@ -439,6 +453,11 @@ vlbm_status ideal_moments_range(vlbm_ctx *c, int d, double *out, int64_t c0, int
 vlbm_status ideal_step(vlbm_ctx *c, int parity);
 bool ideal_double_ok(vlbm_ctx *c);
 vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out);
+
+// launchers (k_double2d.cu): the 2-D two-step pass, single and batched domains
+bool double_2d_ok(vlbm_ctx *c);
+vlbm_status double_2d_prepare(vlbm_ctx *c);
+vlbm_status double_2d(vlbm_ctx *c, const void *in, void *out);
 vlbm_status ideal_moments(vlbm_ctx *c, int d, double *Q_dev);
 vlbm_status ideal_gather(vlbm_ctx *c, int d, const int64_t *cells_dev, int n, double *out_dev);
 vlbm_status ideal_sums(vlbm_ctx *c, int d, double *sums_dev);

@@ -60,6 +60,58 @@ def test_equals_single_steps(V, shape, calls):
     assert np.array_equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("shape,calls", [((2048, 2048), (4, 10)), ((1999, 2311), (41, 8)), ((4099, 1030), (6,))])
+def test_2d_equals_single_steps(V, shape, calls):
+    import torch
+    f0 = fields.ideal_fields(shape, 25, mach=0.5, beta=1.0, cfl=0.1, device=torch.device("cuda"))
+    tau = np.array([0.51, 0.6, 0.55, 0.7, 0.52, 0.8, 0.65, 0.9])
+    src = np.array([1e-7, -2e-7, 3e-7, 0.0, 1e-8, 2e-8, -1e-8, 0.0])
+    p = V.make_params(shape=shape, storage="f32", gamma=f0.gamma, tau=tau, source=src)
+    got, passes = [], []
+    for one in (False, True):
+        with V.Context(p) as ctx:
+            assert V.vlbm_init_fields_device(ctx.ptr, 0, f0.Q.data_ptr()) == V.VLBM_OK
+            before = ctx.launches
+            for n in calls:
+                for _ in range(n if one else 1):
+                    assert ctx.step(1 if one else n) == V.VLBM_OK
+            passes.append(ctx.launches - before)
+            assert ctx.sync() == V.VLBM_OK
+            got.append(populations(V, ctx, shape, 26))
+    assert np.array_equal(got[0], got[1])
+    assert passes[0] < passes[1] == sum(calls)
+
+
+def test_batch_equals_single_steps(V):
+    import torch
+    sides = [(1024, 1024), (64, 64), (31, 33), (512, 700), (128, 130), (1, 90), (90, 1), (800, 1000)]
+    params, Q = [], []
+    for i, shape in enumerate(sides):
+        f0 = fields.ideal_fields(shape, 30 + i, gamma=1.4 + 0.03 * i, mach=0.2, cfl=0.1, k_rho=1, k_u=1, k_b=1,
+                                 device=torch.device("cuda")) if min(shape) > 2 else None
+        if f0 is None:
+            u = fields.uniform_ideal_state(shape, rho=1.1, u=(0.01, 0.02, 0.0), p=0.02, B=(0.01, 0.0, 0.02), gamma=1.5)
+            Q.append(torch.as_tensor(u, device="cuda"))
+        else:
+            Q.append(f0.Q)
+        params.append(V.make_params(shape=shape, storage="f32", gamma=1.4 + 0.03 * i, tau=0.55 + 0.01 * i))
+    got, passes = [], []
+    for one in (False, True):
+        with V.Context(params, batch=True) as ctx:
+            for d, q in enumerate(Q):
+                assert V.vlbm_init_fields_device(ctx.ptr, d, q.data_ptr()) == V.VLBM_OK
+            before = ctx.launches
+            for n in (4, 36, 7):
+                for _ in range(n if one else 1):
+                    assert ctx.step(1 if one else n) == V.VLBM_OK
+            passes.append(ctx.launches - before)
+            assert ctx.sync() == V.VLBM_OK
+            got.append([ctx.populations(np.arange(int(np.prod(s))), d) for d, s in enumerate(sides)])
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+    assert passes[0] < passes[1] == 47
+
+
 def test_refused_second_buffer_takes_single_steps(V):
     """An allocator that has no second buffer to give: every step its own launch, same state."""
     import torch
