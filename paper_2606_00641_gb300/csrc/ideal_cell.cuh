@@ -199,14 +199,14 @@ VLBM_HD __forceinline__ void ideal_collide_f64(C (&f)[8][AxisSet<D>::Q], const C
 // bits: left to the compiler, which products are fused differs from kernel to kernel.
 // relax: a function from lattice to its constants and source terms.  The two directions of an axis get
 // +- omega phi / 2 last, as one rounded value (see relax_lattice).
-template <int D, class W>
-__device__ __forceinline__ void ideal_collide_f32(float (&f)[8][AxisSet<D>::Q], const float gm1, const W &relax,
-                                                  unsigned *flags)
+template <int D, int NL = 8, class W>
+__device__ __forceinline__ void ideal_collide_f32(float (&f)[NL][AxisSet<D>::Q], const float gm1, const W &relax,
+                                                  unsigned *flags, const float inv_tau_m = 0.f)
 {
     constexpr int Q = AxisSet<D>::Q;
-    float q[8];
+    float q[NL];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < NL; ++k) {
         float s = f[k][0];
 #pragma unroll
         for (int i = 1; i < Q; ++i) s = __fadd_rn(s, f[k][i]);
@@ -223,7 +223,7 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[8][AxisSet<D>::Q], 
     const float pt = __fmaf_rn(0.5f, B2, p);
     if (!(q[0] > 0.f) || !(p > 0.f)) raise_flag(flags, kFlagNonPhysical);
     const float Ept = __fadd_rn(q[4], pt);
-    float phi[8][D];
+    float phi[NL][D];
 #pragma unroll
     for (int ax = 0; ax < D; ++ax) {
         phi[0][ax] = m[ax];
@@ -240,10 +240,26 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[8][AxisSet<D>::Q], 
         }
         phi[4][ax] = __fmaf_rn(Ept, u[ax], -__fmul_rn(B[ax], uB));
     }
+    float ndiv = 0.f;  // Powell form: -div B
+    if constexpr (NL == 9) {
+        ndiv = __fmul_rn(-q[8], inv_tau_m);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+        for (int ax = 0; ax < D; ++ax) phi[8][ax] = __fmaf_rn(q[8], u[ax], -B[ax]);
+    }
+#pragma unroll
+    for (int k = 0; k < NL; ++k) {
         const RelaxSource r = relax(k);
-        const float A0 = __fmaf_rn(r.ow0, q[k], r.src0), A1 = __fmaf_rn(r.ow1, q[k], r.src1);
+        float A0 = __fmaf_rn(r.ow0, q[k], r.src0), A1 = __fmaf_rn(r.ow1, q[k], r.src1);
+        if constexpr (NL == 9) {
+            if (k > 0) {  // S = -(div B)(0, B, u.B, u) and, for D, -D / tau_M = -div B
+                const float S = k == 8   ? ndiv
+                                : k >= 5 ? __fmul_rn(ndiv, u[k >= 5 && k < 8 ? k - 5 : 0])
+                                : k == 4 ? __fmul_rn(ndiv, uB)
+                                         : __fmul_rn(ndiv, B[k >= 1 && k < 4 ? k - 1 : 0]);
+                A0 = __fmaf_rn(ExactWeights<D, float>::w0, S, A0);
+                A1 = __fmaf_rn(ExactWeights<D, float>::w1, S, A1);
+            }
+        }
         f[k][0] = __fmaf_rn(r.omc, f[k][0], A0);
 #pragma unroll
         for (int ax = 0; ax < D; ++ax) {

@@ -103,7 +103,10 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
         }
 
     const auto &omega = step_omega(a);
-    if constexpr (NL == 9) {
+    if constexpr (NL == 9 && sizeof(C) == 4) {
+        ideal_collide_f32<D, 9>(
+            f, a.gm1, [&](int k) { return relax_source<D>(a.omega[k], a.src0[k], a.src1[k]); }, a.flags, a.inv_tau_m);
+    } else if constexpr (NL == 9) {
         powell_collide<D, C>(f, a.gm1, omega, a.src0, a.src1, a.inv_tau_m, a.flags);
     } else if constexpr (HOM) {
         const float *sp = a.solid + cell;
@@ -412,11 +415,11 @@ __global__ void __launch_bounds__(kPairThreads, 6) k_ideal_step_pairs(const Idea
     }
 }
 
-// Two steps of the plain 3-D FP32 form in one pass: an even and an odd one, from parity 0
+// Two steps of the plain 3-D FP32 form (or Powell's, NL = 9) in one pass: an even and an odd one, from parity 0
 // in one buffer to parity 0 in another, every population read once and written once for
 // both.  One step is bound by HBM (448 B a cell at the copy rate), so this is where a
-// large box gains.  A CTA takes a column of up to kDblX x kDblY cells over kDblZ planes
-// and walks up it.  Per plane:
+// large box gains.  A CTA takes a column of up to kDblX x kDblY cells over some
+// sixteen planes and walks up it.  Per plane:
 //   1. every thread (32 x (kDblY + 2): the column and a rim one cell wide) loads its
 //      cell's populations and collides them (step 1);
 //   2. what step 1 sends along x and y goes to the neighbours through shared memory
@@ -436,30 +439,32 @@ __global__ void __launch_bounds__(kPairThreads, 6) k_ideal_step_pairs(const Idea
 // registers) 13.83 at 512^3 but 0.259 at 128^3; 14 rows, one CTA per SM, 17.0; 32 planes
 // 14.2 at 512^3; three CTAs of 96 registers 31.4 (spills); the next plane's populations
 // staged by cp.async 17.4 or more (4-byte copies); the z and rest values in shared memory 16.9.
-constexpr int kDblX = 30, kDblY = 6, kDblZ = 16;
-constexpr int kDblThreads = 32 * (kDblY + 2);
-constexpr int kDblSmem = 3 * 32 * kDblThreads * (int)sizeof(float);
+constexpr int kDblX = 30;
+template <int NL> constexpr int kDblY = NL == 8 ? 6 : 4;  // nine lattices: 168 registers, so 192 threads
+template <int NL> constexpr int kDblThreads = 32 * (kDblY<NL> + 2);
+template <int NL> constexpr int kDblSmem = 3 * 4 * NL * kDblThreads<NL> * (int)sizeof(float);
 
 struct DoubleArgs {
     const float *in;
     float *out;
     int nx, ny, nz;
     int tile_x, tiles_x, tiles_y;  // columns of tile_x <= kDblX cells
+    int tile_z;                    // and so many planes
     int64_t stride;
-    float gm1;
-    RelaxSource relax[8];
+    float gm1, inv_tau_m;
+    RelaxSource relax[9];
     unsigned *flags;
 };
 
-__global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArgs a)
+template <int NL> __global__ void __launch_bounds__(kDblThreads<NL>, 2) k_ideal_double(const DoubleArgs a)
 {
     extern __shared__ float exchange[];  // [plane % 3][lattice and direction 1 .. 4][thread]
-    constexpr int NT = kDblThreads;
+    constexpr int NT = kDblThreads<NL>, PLANE = 4 * NL * NT;
     const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5;
     const int tx = blockIdx.x % a.tiles_x, ty = blockIdx.x / a.tiles_x % a.tiles_y,
               tz = blockIdx.x / a.tiles_x / a.tiles_y;
-    const int x0 = tx * a.tile_x, y0 = ty * kDblY, z0 = tz * kDblZ;
-    const int xe = min(x0 + a.tile_x, a.nx), ye = min(y0 + kDblY, a.ny), ze = min(z0 + kDblZ, a.nz);
+    const int x0 = tx * a.tile_x, y0 = ty * kDblY<NL>, z0 = tz * a.tile_z;
+    const int xe = min(x0 + a.tile_x, a.nx), ye = min(y0 + kDblY<NL>, a.ny), ze = min(z0 + a.tile_z, a.nz);
     int x = x0 - 1 + lx, y = y0 - 1 + ly;
     const bool first = x <= xe && y <= ye;                            // takes part in step 1
     const bool second = lx >= 1 && ly >= 1 && x < xe && y < ye;       // and in step 2
@@ -470,31 +475,31 @@ __global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArg
     const uint32_t xm = x > 0 ? at - 1 : at + row - 1, xp = x + 1 < a.nx ? at + 1 : at + 1 - row;
     const uint32_t ym = y > 0 ? at - row : at + plane - row, yp = y + 1 < a.ny ? at + row : at + row - plane;
     auto relax = [&](int k) { return a.relax[k]; };
-    float rest[8], up1[8], up2[8];  // step 1: at rest on the plane below; sent up from it and from the one below that
+    float rest[NL], up1[NL], up2[NL];  // step 1: at rest on the plane below; sent up from it and from the one below that
 #pragma unroll
-    for (int k = 0; k < 8; ++k) rest[k] = up1[k] = up2[k] = 0.f;
+    for (int k = 0; k < NL; ++k) rest[k] = up1[k] = up2[k] = 0.f;
     int buf = 0;
     for (int z = z0 - 1; z <= ze; ++z) {
-        float f[8][7];
-        float *mine = exchange + buf * 32 * NT + tid;
-        const float *below = exchange + (buf == 0 ? 2 : buf - 1) * 32 * NT + tid;
+        float f[NL][7];
+        float *mine = exchange + buf * PLANE + tid;
+        const float *below = exchange + (buf == 0 ? 2 : buf - 1) * PLANE + tid;
         buf = buf == 2 ? 0 : buf + 1;
         if (first) {
             const uint32_t zc = (uint32_t)(z < 0 ? z + a.nz : (z >= a.nz ? z - a.nz : z));
             const float *p = a.in + (at + plane * zc);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
+            for (int k = 0; k < NL; ++k)
 #pragma unroll
                 for (int i = 0; i < 7; ++i) f[k][i] = p[(int64_t)(k * 7 + i) * a.stride];
-            ideal_collide_f32<3>(f, a.gm1, relax, a.flags);
+            ideal_collide_f32<3, NL>(f, a.gm1, relax, a.flags, a.inv_tau_m);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
+            for (int k = 0; k < NL; ++k)
 #pragma unroll
                 for (int i = 1; i < 5; ++i) mine[(k * 4 + i - 1) * NT] = f[k][i];
             // what step 2 of the plane below gets along z and from its own cell; f[k][6] is
             // already what this plane sends down
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < NL; ++k) {
                 const float r = f[k][0], u = f[k][5];
                 f[k][0] = rest[k];
                 f[k][5] = up2[k];
@@ -508,13 +513,13 @@ __global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArg
         __syncthreads();
         if (z > z0 && second) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
+            for (int k = 0; k < NL; ++k) {
                 f[k][1] = below[(k * 4 + 0) * NT - 1];
                 f[k][2] = below[(k * 4 + 1) * NT + 1];
                 f[k][3] = below[(k * 4 + 2) * NT - 32];
                 f[k][4] = below[(k * 4 + 3) * NT + 32];
             }
-            ideal_collide_f32<3>(f, a.gm1, relax, a.flags);
+            ideal_collide_f32<3, NL>(f, a.gm1, relax, a.flags, a.inv_tau_m);
             const int zo = z - 1;
             const uint32_t pz = plane * (uint32_t)zo;
             const uint32_t pp = plane * (uint32_t)(zo + 1 < a.nz ? zo + 1 : 0);
@@ -524,7 +529,7 @@ __global__ void __launch_bounds__(kDblThreads, 2) k_ideal_double(const DoubleArg
             for (int i = 0; i < 7; ++i) {
                 float *o = a.out + to[i];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) o[(int64_t)(k * 7 + i) * a.stride] = f[k][i];
+                for (int k = 0; k < NL; ++k) o[(int64_t)(k * 7 + i) * a.stride] = f[k][i];
             }
         }
     }
@@ -1119,54 +1124,70 @@ template <int D, class S> struct OpenF {
 
 vlbm_status ideal_step(vlbm_ctx *c, int parity) { return dispatch<StepF>(c, parity); }
 
-// Columns of the two-step pass over a box.
-static void double_tiles(const Domain &d, int &tile_x, int &tiles_x, int &tiles_y, int &tiles_z)
+// Columns of the two-step pass over a box, and the share of wanted cells among those that
+// all waves of CTAs could produce, rims and end planes included.  Of 12 to 18 planes a
+// column the number with the largest share (more drift apart, see above).
+template <int NL> static double double_tiles(const Domain &d, int slots, DoubleArgs &a, int64_t &ctas)
 {
-    tiles_x = (d.nx + kDblX - 1) / kDblX;
-    tile_x = (d.nx + tiles_x - 1) / tiles_x;
-    tiles_y = (d.ny + kDblY - 1) / kDblY;
-    tiles_z = (d.nz + kDblZ - 1) / kDblZ;
+    a.tiles_x = (d.nx + kDblX - 1) / kDblX;
+    a.tile_x = (d.nx + a.tiles_x - 1) / a.tiles_x;
+    a.tiles_y = (d.ny + kDblY<NL> - 1) / kDblY<NL>;
+    double best = 0.0;
+    for (int z : {16, 18, 17, 15, 14, 13, 12}) {
+        const int64_t n = (int64_t)a.tiles_x * a.tiles_y * ((d.nz + z - 1) / z);
+        const int64_t waves = (n + slots - 1) / slots;
+        const double share = (double)d.ncell / ((double)waves * slots * kDblX * kDblY<NL> * (z + 2));
+        if (share > 1.02 * best) {
+            best = share;
+            a.tile_z = z;
+            ctas = n;
+        }
+    }
+    return best;
 }
 
-// Where the two-step pass is taken: plain 3-D FP32 boxes whose populations exceed L2
-// (below, a step is not bound by HBM) and whose columns fill the CTA slots well: of the
-// cells that all waves of CTAs could produce, rims and end planes included, at least 0.7
-// are wanted cells.  The gain is proportional to that share: 1.27 at 512^3 (0.84), 1.17 at
-// 128^3 (0.71), 0.91 at 96^3 (0.45).
+template <int NL> static int double_slots_of_device()
+{
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaFuncSetAttribute(k_ideal_double<NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDblSmem<NL>) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ideal_double<NL>, kDblThreads<NL>, kDblSmem<NL>) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        per_sm = 0;
+    }
+    return per_sm > 0 ? sms * per_sm : -1;
+}
+
+// Where the two-step pass is taken: plain (or Powell) 3-D FP32 boxes whose populations
+// exceed L2 (below, a step is not bound by HBM) and whose columns fill the CTA slots well,
+// a share of at least 0.7.  The gain is proportional to the share: 1.27 at 512^3 (0.84),
+// 1.17 at 128^3 (0.71), 0.91 at 96^3 (0.45); Powell 90 x 130 x 150 (0.80) 1.28.
 bool ideal_double_ok(vlbm_ctx *c)
 {
-    if (c->batched || c->model != VLBM_IDEAL || c->nlat != 8 || c->dim != 3 || c->storage != VLBM_F32 || c->slab ||
-        c->closure || c->solid || any_open_face(c))
+    if (c->batched || (c->model != VLBM_IDEAL && c->model != VLBM_IDEAL_POWELL) || c->dim != 3 ||
+        c->storage != VLBM_F32 || c->slab || c->closure || c->solid || any_open_face(c))
         return false;
     const Domain &d = c->dom[0];
     if (c->pop_bytes < (size_t(128) << 20) || d.ncell > (int64_t(1) << 30)) return false;
-    if (c->double_slots == 0) {
-        int dev = 0, sms = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (cudaFuncSetAttribute(k_ideal_double, cudaFuncAttributeMaxDynamicSharedMemorySize, kDblSmem) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ideal_double, kDblThreads, kDblSmem) !=
-                cudaSuccess) {
-            cudaGetLastError();
-            per_sm = 0;
-        }
-        c->double_slots = per_sm > 0 ? sms * per_sm : -1;
-    }
+    const bool powell = c->nlat == 9;
+    if (c->double_slots == 0) c->double_slots = powell ? double_slots_of_device<9>() : double_slots_of_device<8>();
     if (c->double_slots < 0) return false;
-    int tile_x, tiles_x, tiles_y, tiles_z;
-    double_tiles(d, tile_x, tiles_x, tiles_y, tiles_z);
-    const int64_t ctas = (int64_t)tiles_x * tiles_y * tiles_z;
-    const int64_t waves = (ctas + c->double_slots - 1) / c->double_slots;
-    const double could = (double)waves * c->double_slots * (kDblX * kDblY) * (kDblZ + 2);
-    return ctas <= 0x7FFFFFFF && (double)d.ncell >= 0.7 * could;
+    DoubleArgs a{};
+    int64_t ctas = 0;
+    const double share = powell ? double_tiles<9>(d, c->double_slots, a, ctas) : double_tiles<8>(d, c->double_slots, a, ctas);
+    return share >= 0.7 && ctas <= 0x7FFFFFFF;
 }
 
-// One even and one odd step of every cell, `in` (parity 0) to `out` (parity 0).
-vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out)
+template <int NL> static vlbm_status double_t(vlbm_ctx *c, const void *in, void *out)
 {
     const Domain &d = c->dom[0];
     const IdealArgs<float> s = make_step_args<float>(c);
     DoubleArgs a{};
+    int64_t ctas = 0;
+    double_tiles<NL>(d, c->double_slots, a, ctas);
     a.in = static_cast<const float *>(in);
     a.out = static_cast<float *>(out);
     a.nx = d.nx;
@@ -1174,13 +1195,18 @@ vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out)
     a.nz = d.nz;
     a.stride = d.stride;
     a.gm1 = s.gm1;
-    for (int k = 0; k < 8; ++k) a.relax[k] = relax_source<3>(s.omega[k], s.src0[k], s.src1[k]);
+    a.inv_tau_m = s.inv_tau_m;
+    for (int k = 0; k < NL; ++k) a.relax[k] = relax_source<3>(s.omega[k], s.src0[k], s.src1[k]);
     a.flags = c->d_flags;
-    int tiles_z;
-    double_tiles(d, a.tile_x, a.tiles_x, a.tiles_y, tiles_z);
-    k_ideal_double<<<(unsigned)(a.tiles_x * a.tiles_y * tiles_z), kDblThreads, kDblSmem, c->stream>>>(a);
+    k_ideal_double<NL><<<(unsigned)ctas, kDblThreads<NL>, kDblSmem<NL>, c->stream>>>(a);
     c->launches++;
     return cuda_check(c, cudaGetLastError(), "two-step launch");
+}
+
+// One even and one odd step of every cell, `in` (parity 0) to `out` (parity 0).
+vlbm_status ideal_double(vlbm_ctx *c, const void *in, void *out)
+{
+    return c->nlat == 9 ? double_t<9>(c, in, out) : double_t<8>(c, in, out);
 }
 
 vlbm_status ideal_step_corrected(vlbm_ctx *c, int parity, const float *dphi)

@@ -60,6 +60,28 @@ def test_equals_single_steps(V, shape, calls):
     assert np.array_equal(got[0], got[1])
 
 
+@pytest.mark.parametrize("shape,calls", [((90, 130, 150), (40, 5)), ((121, 141, 178), (6, 8))])
+def test_powell_equals_single_steps(V, shape, calls):
+    import torch
+    f0 = fields.ideal_fields(shape, 28, mach=0.5, beta=1.0, cfl=0.2, device=torch.device("cuda"))
+    Q = torch.cat([f0.Q, 1e-3 * (f0.Q[:1] - 1.0)])
+    p = V.make_params(model=V.VLBM_IDEAL_POWELL, shape=shape, storage="f32", gamma=f0.gamma, tau=0.55, tau_d=0.6,
+                      tau_m=1.5)
+    got, passes = [], []
+    for one in (False, True):
+        with V.Context(p) as ctx:
+            assert V.vlbm_init_fields_device(ctx.ptr, 0, Q.data_ptr()) == V.VLBM_OK
+            before = ctx.launches
+            for n in calls:
+                for _ in range(n if one else 1):
+                    assert ctx.step(1 if one else n) == V.VLBM_OK
+            passes.append(ctx.launches - before)
+            assert ctx.sync() == V.VLBM_OK
+            got.append(populations(V, ctx, shape, 29))
+    assert np.array_equal(got[0], got[1])
+    assert passes[0] < passes[1] == sum(calls)
+
+
 @pytest.mark.parametrize("shape,calls", [((2048, 2048), (4, 10)), ((1999, 2311), (41, 8)), ((4099, 1030), (6,))])
 def test_2d_equals_single_steps(V, shape, calls):
     import torch
