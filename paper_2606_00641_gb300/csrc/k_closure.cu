@@ -1049,13 +1049,16 @@ __global__ void __launch_bounds__(256) k_part_sums(const __grid_constant__ PartS
 // is a GEMM whose reduction runs over the cells.  Both operands are read in
 // their natural cell-major layout (channels contiguous), i.e. as MN-major
 // operands, from planes staged in shared memory:
-//   A (M = 128 rows) = 4 z-offsets x 4 slots x 8 channels.  Row z-offset h is
-//     the tap dz = h (h = 3 is computed and discarded).  With 32 input channels
-//     the slots are the 4 channel blocks and there is one accumulator per
-//     (dy, dx); with 8 input channels the slots hold copies of the halo
-//     shifted by dx = 0, 1, 2 (slot 3 discarded) and there is one accumulator
-//     per dy.  A tap (dy, dx) is an address offset into the staged planes.
-//   B (N = 32) = the output-channel gradients of the tile's cells.
+//   32 input channels: A (M = 128 rows) = 4 z-offsets x 32 channels of the tile's own
+//     cells (row z-offset h is the tap dz = h; h = 3 is computed and discarded).  The x and
+//     y shifts are put on the other operand: B (N = 96) = the output-channel gradients
+//     staged three times, shifted by dx = -1, 0, 1, and a tap dy is a row offset into them:
+//     three accumulators of 96 columns.  An MMA costs about 60 cycles for any N up to 96,
+//     so this takes a third of the 144 a tile that one accumulator per (dy, dx) with N = 32
+//     took: 52 -> 37 us at 64^3; staging binds now.
+//   8 input channels: A = 4 z-offsets x 4 slots x 8 channels, the slots copies of the halo
+//     shifted by dx = 0, 1, 2 (slot 3 discarded), B (N = 32) the gradients of the tile's
+//     cells, one accumulator per dy, a tap dy an address offset into the staged planes.
 // Tiles of 8 x 16 x kWgZ cells; persistent CTAs (one per SM: the two staging
 // buffers take more than half of the shared memory) accumulate all their
 // tiles in TMEM while the next tile is staged with cp.async (warps 0-7; warp
@@ -1067,15 +1070,25 @@ constexpr int kWgZ = 2;
 constexpr int kWgThreads = 288;  // warps 0-7 stage, warp 8 issues the MMAs, warps 0-2 drain
 constexpr int kWgStage = 256;
 
-template <int CIN>
-struct WgLayout {
-    static constexpr int PW = CIN == 32 ? 10 : 8;  // staged row width in cells
-    static constexpr int S2D = 18 * PW * 16;       // bytes per (z plane, slot)
+template <int CIN> struct WgLayout;
+template <> struct WgLayout<32> {
+    static constexpr int S2D = 128 * 16;             // bytes per (z plane, channel block) of A
+    static constexpr int ABYTES = (kWgZ + 3) * 4 * S2D;
+    static constexpr int GZ = 18 * 8 * 16;           // bytes per z plane of B: 18 rows of 8 cells
+    static constexpr int GROUP = kWgZ * GZ;          // per (dx, channel block)
+    static constexpr int GBYTES = 12 * GROUP;
+    static constexpr int BUF = ABYTES + GBYTES;
+    static constexpr int NACC = 3, N = 96;
+    static constexpr int COLS = 512;                 // TMEM columns (power of two >= N * NACC)
+};
+template <> struct WgLayout<8> {
+    static constexpr int PW = 8;                     // staged row width in cells
+    static constexpr int S2D = 18 * PW * 16;         // bytes per (z plane, slot)
     static constexpr int ABYTES = (kWgZ + 3) * 4 * S2D;
     static constexpr int GBYTES = 4 * kWgZ * 128 * 16;
     static constexpr int BUF = ABYTES + GBYTES;
-    static constexpr int NACC = CIN == 32 ? 9 : 3;
-    static constexpr int COLS = CIN == 32 ? 512 : 128;  // TMEM columns (power of two >= 32 * NACC)
+    static constexpr int NACC = 3, N = 32;
+    static constexpr int COLS = 128;
 };
 
 template <int CIN>
@@ -1116,46 +1129,50 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const bf16 *__restrict_
         const int tx = tile % tiles_x, ty = (tile / tiles_x) % tiles_y, tz = tile / (tiles_x * tiles_y);
         const int x0 = tx * 8, y0 = ty * 16, z0 = tz * kWgZ;
         const uint32_t abase = s_base + (uint32_t)(b * L::BUF), gbase = abase + L::ABYTES;
-        constexpr int NA = CIN == 32 ? (kWgZ + 2) * 4 * 18 * 10 : (kWgZ + 2) * 3 * 18 * 8;
-        for (int idx = tid; idx < NA; idx += kWgStage) {
-            int slot, bx, by, h, sx;
-            if (CIN == 32) {  // slot = channel block; consecutive threads read one cell's 64 bytes
-                slot = idx & 3;
-                const int c = idx >> 2;
-                bx = c % 10;
-                by = (c / 10) % 18;
-                h = c / 180;
-                sx = bx;
-            } else {          // slot = x shift
-                bx = idx & 7;
-                const int r = idx >> 3;
-                by = r % 18;
-                slot = (r / 18) % 3;
-                h = r / 54;
-                sx = bx + slot;
-            }
-            int gx = x0 - 1 + sx, gy = y0 - 1 + by, gzz = z0 - 1 + h;
-            gx += gx < 0 ? nx : (gx >= nx ? -nx : 0);
-            gy += gy < 0 ? ny : (gy >= ny ? -ny : 0);
-            gzz += gzz < 0 ? nz : (gzz >= nz ? -nz : 0);
-            const size_t cell = (size_t)gx + (size_t)nx * gy + (size_t)plane * gzz;
-            const uint32_t dst = abase + (uint32_t)((((h * 4 + slot) * 18 + by) * L::PW + bx) * 16);
-            const bf16 *src = act + ((size_t)(CIN == 32 ? slot : 0) * Ncell + cell) * 8;
+        auto wrap = [](int v, int n) { return v + (v < 0 ? n : (v >= n ? -n : 0)); };
+        auto copy = [](uint32_t dst, const bf16 *src) {
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-        }
-        for (int idx = tid; idx < 4 * kWgZ * 128; idx += kWgStage) {
-            const int cbo = idx & 3, c = idx >> 2;  // c = zz * 128 + y * 8 + x
-            const size_t cell = (size_t)(x0 + (c & 7)) + (size_t)nx * (y0 + ((c >> 3) & 15)) +
-                                (size_t)plane * (z0 + (c >> 7));
-            const uint32_t dst = gbase + (uint32_t)((cbo * kWgZ * 128 + c) * 16);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gz + ((size_t)cbo * Ncell + cell) * 8)
-                         : "memory");
+        };
+        if constexpr (CIN == 32) {
+            // A: planes z0 - 1 .. z0 + kWgZ of the tile's cells; thread = (cell, half of the blocks)
+            const int cell = tid & 127, cb0 = tid >> 7;
+            const int x = x0 + (cell & 7), y = y0 + (cell >> 3);
+#pragma unroll
+            for (int h = 0; h < kWgZ + 2; ++h) {
+                const size_t at = (size_t)x + (size_t)nx * y + (size_t)plane * wrap(z0 - 1 + h, nz);
+#pragma unroll
+                for (int cb = cb0; cb < 4; cb += 2)
+                    copy(abase + (uint32_t)((h * 4 + cb) * L::S2D + cell * 16), act + ((size_t)cb * Ncell + at) * 8);
+            }
+            // B: rows y0 - 1 .. y0 + 16, three copies with x - dx, dx = s - 1
+            for (int idx = tid; idx < kWgZ * 18 * 8 * 3; idx += kWgStage) {
+                const int bx = idx & 7, r = idx >> 3, by = r % 18, q = r / 18, s = q % 3, zz = q / 3;
+                const size_t at = (size_t)wrap(x0 + bx + 1 - s, nx) + (size_t)nx * wrap(y0 - 1 + by, ny) +
+                                  (size_t)plane * (z0 + zz);
+                const uint32_t dst = gbase + (uint32_t)(s * 4 * L::GROUP + zz * L::GZ + (by * 8 + bx) * 16);
+#pragma unroll
+                for (int cb = 0; cb < 4; ++cb)
+                    copy(dst + (uint32_t)(cb * L::GROUP), gz + ((size_t)cb * Ncell + at) * 8);
+            }
+        } else {
+            for (int idx = tid; idx < (kWgZ + 2) * 3 * 18 * 8; idx += kWgStage) {
+                const int bx = idx & 7, r = idx >> 3, by = r % 18, slot = (r / 18) % 3, h = r / 54;
+                const size_t cell = (size_t)wrap(x0 - 1 + bx + slot, nx) + (size_t)nx * wrap(y0 - 1 + by, ny) +
+                                    (size_t)plane * wrap(z0 - 1 + h, nz);
+                copy(abase + (uint32_t)((((h * 4 + slot) * 18 + by) * L::PW + bx) * 16), act + cell * 8);
+            }
+            for (int idx = tid; idx < 4 * kWgZ * 128; idx += kWgStage) {
+                const int cbo = idx & 3, c = idx >> 2;  // c = zz * 128 + y * 8 + x
+                const size_t cell = (size_t)(x0 + (c & 7)) + (size_t)nx * (y0 + ((c >> 3) & 15)) +
+                                    (size_t)plane * (z0 + (c >> 7));
+                copy(gbase + (uint32_t)((cbo * kWgZ * 128 + c) * 16), gz + ((size_t)cbo * Ncell + cell) * 8);
+            }
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
 
-    // MN-major A and B (bits 15, 16), BF16 in, FP32 accumulate, M = 128, N = 32
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((32u >> 3) << 17) |
+    // MN-major A and B (bits 15, 16), BF16 in, FP32 accumulate, M = 128
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (((uint32_t)L::N >> 3) << 17) |
                            ((128u >> 4) << 24);
     uint32_t phase = 0;
     bool ok = true, first = true;
@@ -1171,16 +1188,19 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const bf16 *__restrict_
             const uint32_t abase = s_base + (uint32_t)(b * L::BUF), gbase = abase + L::ABYTES;
             for (int zz = 0; zz < kWgZ; ++zz)
                 for (int ks = 0; ks < 8; ++ks) {  // two tile rows of 8 cells per K step
-                    const uint64_t db = tc_desc(gbase + (uint32_t)(zz * 2048 + ks * 256), 128, kWgZ * 128 * 16);
                     const uint32_t acc = !(first && zz == 0 && ks == 0);
-                    for (int j = 0; j < L::NACC; ++j) {
-                        const int dy = CIN == 32 ? j / 3 : j, dx = CIN == 32 ? j % 3 : 0;
-                        const uint32_t a_addr =
-                            abase + (uint32_t)(zz * 4 * L::S2D + ((2 * ks + dy) * L::PW + dx) * 16);
-                        const uint64_t da = tc_desc(a_addr, L::PW * 16, L::S2D);
-                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-                                     ::"r"(tmem + (uint32_t)(32 * j)), "l"(da), "l"(db), "r"(idesc), "r"(acc));
+#pragma unroll
+                    for (int j = 0; j < L::NACC; ++j) {  // tap dy = j - 1
+                        uint64_t da, db;
+                        if constexpr (CIN == 32) {
+                            da = tc_desc(abase + (uint32_t)(zz * 4 * L::S2D + ks * 256), 128, L::S2D);
+                            db = tc_desc(gbase + (uint32_t)(zz * L::GZ + (2 * ks + 2 - j) * 128), 128, L::GROUP);
+                        } else {
+                            da = tc_desc(abase + (uint32_t)(zz * 4 * L::S2D + (2 * ks + j) * L::PW * 16), L::PW * 16,
+                                         L::S2D);
+                            db = tc_desc(gbase + (uint32_t)(zz * 2048 + ks * 256), 128, kWgZ * 128 * 16);
+                        }
+                        tc_mma(tmem + (uint32_t)(L::N * j), da, db, idesc, acc);
                     }
                 }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mb));
@@ -1189,10 +1209,18 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const bf16 *__restrict_
         const int next = tile + (int)gridDim.x;
         if (next < ntiles && warp < 8) stage(next, b ^ 1);
         if (warp < 8) {  // this tile's output gradients (channel lane) from the staged planes
-            const unsigned char *g = smem + b * L::BUF + L::ABYTES + (lane >> 3) * (kWgZ * 128 * 16) + (lane & 7) * 2;
+            const unsigned char *g = smem + b * L::BUF + L::ABYTES + (lane & 7) * 2;
+            if constexpr (CIN == 32) {  // the unshifted copy, without its y halo
+                g += (4 + (lane >> 3)) * L::GROUP + 8 * 16;
 #pragma unroll 8
-            for (int c = warp; c < kWgZ * 128; c += 8)
-                bsum += __bfloat162float(*reinterpret_cast<const bf16 *>(g + c * 16));
+                for (int c = warp; c < kWgZ * 128; c += 8)
+                    bsum += __bfloat162float(*reinterpret_cast<const bf16 *>(g + (c >> 7) * L::GZ + (c & 127) * 16));
+            } else {
+                g += (lane >> 3) * (kWgZ * 128 * 16);
+#pragma unroll 8
+                for (int c = warp; c < kWgZ * 128; c += 8)
+                    bsum += __bfloat162float(*reinterpret_cast<const bf16 *>(g + c * 16));
+            }
         }
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -1226,7 +1254,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_tc(const bf16 *__restrict_
     }
     if (ok && warp < 3) {  // warp h reads TMEM lanes of z-offset h = dz; warp 3 holds discarded rows
         float *dst = part + (size_t)blockIdx.x * pstride;
-        for (int j = 0; j < L::NACC; ++j) {
+        for (int j = 0; j < L::NACC * (L::N / 32); ++j) {  // CIN = 32: j = 3 dy + dx
             uint32_t r[32];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(32 * j);
             asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
