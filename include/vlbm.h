@@ -198,8 +198,9 @@ vlbm_status vlbm_init_fields_device(vlbm_ctx *ctx, int domain, const double *Q_d
 /* Enqueue n >= 0 time steps of Eq. 2 on every domain: one fused
  * collide-and-stream kernel per step (in-place AA pattern), asynchronous.
  * Large plain ideal F32 boxes (and batches) take four steps at a time in two kernels of
- * two steps each, bit for bit the same populations, in calls of n >= 4 that
- * begin at an even step count; the first such call allocates a second buffer
+ * two steps each, bit for bit the same populations, in calls of n >= 4 (from an
+ * odd step count after one single step, in the steps past whole runs of 32 on an
+ * own stream); the first such call allocates a second buffer
  * of vlbm_population_bytes (kept until vlbm_destroy), if the populations are at
  * most a sixth of the device's memory and a third of what is free; without it,
  * or on a stream under capture that has none yet, every step is one kernel.

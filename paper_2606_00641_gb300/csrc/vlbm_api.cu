@@ -250,9 +250,8 @@ void ensure_second_buffer(vlbm_ctx *c)
 
 // Launches the next of `left` steps from `parity`: four at once by two two-step passes,
 // out to the second buffer and back, where that pass applies (the populations are in the
-// first buffer whenever a call returns); else one.  Returns how many in *taken.  The
-// caller allows pairs where its run of steps begins at an even step count; a run that
-// begins at an odd one keeps its launch per step, as vlbm_launch_count has reported it.
+// first buffer whenever a call returns); else one.  Returns how many in *taken.  The pass
+// begins at an even parity: a run from an odd step count takes one single step first.
 vlbm_status launch_next(vlbm_ctx *c, bool pairs, int parity, int left, int *taken)
 {
     if (pairs && c->pop2 && parity == 0 && left >= 4 && double_ok(c)) {
@@ -622,8 +621,12 @@ vlbm_status vlbm_step(vlbm_ctx *c, int n)
             return fail(c, VLBM_ERR_ARG, "one face of an axis is open and the other periodic");
     const bool graphs = c->stream != nullptr && c->stream != cudaStreamLegacy &&
                         c->stream != cudaStreamPerThread;
-    const bool pairs = (c->step & 1) == 0;
-    if (pairs && n >= 4) ensure_second_buffer(c);
+    // Steps that four-step passes may take: all from an even step count.  From an odd one
+    // a captured graph keeps its launch per step (a graph is one parity's whole run of
+    // steps), and the launches outside graphs take one single step and then passes:
+    // 512^3, 20 steps from step 5: 8.86 -> 7.31 ms a step.
+    const int odd = (int)(c->step & 1);
+    if ((odd && graphs ? n % kGraphLen : n) >= 4 + odd) ensure_second_buffer(c);
     int left = n;
     while (left > 0) {
         if (graphs && left >= kGraphLen) {
@@ -639,7 +642,7 @@ vlbm_status vlbm_step(vlbm_ctx *c, int n)
             }
         }
         int taken = 0;
-        vlbm_status s = launch_next(c, pairs, (int)(c->step & 1), left, &taken);
+        vlbm_status s = launch_next(c, true, (int)(c->step & 1), left, &taken);
         if (s != VLBM_OK) return s;
         c->step += taken;
         left -= taken;

@@ -51,10 +51,10 @@ def test_equals_single_steps(V, shape, calls):
             passes = ctx.launches - before
             assert ctx.sync() == V.VLBM_OK
             got.append(populations(V, ctx, shape, 22))
-            # a launch per step, or two per four steps in calls that begin at an even step count
+            # a launch per step, or two per four steps after a single one from an odd step count
             want, at = 0, 0
             for n in calls:
-                want += n // 4 * 2 + n % 4 if at % 2 == 0 else n
+                want += at % 2 + (n - at % 2) // 4 * 2 + (n - at % 2) % 4
                 at += n
             assert passes == (sum(calls) if one else want)
     assert np.array_equal(got[0], got[1])
