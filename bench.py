@@ -4,10 +4,11 @@
 Workload (default): 3-D ideal compressible MHD, 512^3 periodic cells, 8
 conserved fields each on its own D3Q7 lattice (56 populations per cell),
 FP32 storage and arithmetic, seeded random-phase fields (k <= 4, peak Mach 2,
-beta 1, CFL 0.2, tau 0.51).  One step = one launch of the fused kernel over
-all cells.  Metric: GLUPS (10^9 cell updates per second, whole job) and the
-fraction of the HBM roofline (448 algorithmic bytes per cell update: every
-population read once and written once).
+beta 1, CFL 0.2, tau 0.51).  A launch advances all cells by one step, or by two
+(two-step passes, two per four steps where vlbm_step can take them).  Metric:
+GLUPS (10^9 cell updates per second, whole job) and the fraction of the HBM
+roofline (448 algorithmic bytes per cell and launch: every population read once
+and written once).
 
 Printed: one JSON line on rank 0.  ``--impl reference`` times the CPU oracle
 (plain FP64 C) on the host cores on a bounded sample of the same workload.
@@ -39,24 +40,26 @@ BYTES_PER_POP = {"f64": 8, "f32": 4, "f16dev": 2, "bf16dev": 2}
 # DRAM bytes (read + write) per cell update of the step kernel, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of a 256^3 launch of
 # each parity, mean of the two parities, taken after the last change to that
-# kernel's source: f32 7,457,219 kB and f16dev 3,705,818 kB per 16,777,216-cell
-# launch.  Traffic grows in proportion to the cells, so a full launch is this
+# kernel's source: f32 7,457,546 kB and f16dev 3,703,464 kB per 16,777,216-cell
+# launch, and 8,004,037 kB per two-step pass (f32).  Traffic grows in proportion to the cells, so a full launch is this
 # times the cells.  Set an entry to None whenever that kernel changes until it
 # is re-captured.
-MEASURED_DRAM_BYTES_PER_CELL = {"f32": 7457219e3 / 16777216, "f16dev": 3705818e3 / 16777216}
+MEASURED_DRAM_BYTES_PER_CELL = {"f32": 7457546e3 / 16777216, "f16dev": 3703464e3 / 16777216}
+MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS = {"f32": 8004037e3 / 16777216}
 # FP64 operations per cell update of the FP64 step kernels (k_ideal_step<D,double>),
 # from one ncu capture of each parity: (dadd + dmul + 2 dfma thread instructions,
 # smsp__sass_thread_inst_executed_op_d{add,mul,fma}_pred_on.sum) / cells, mean of
-# the two parities.  3-D (128^3): even 90 + 42 + 2 x 152 = 436, odd 114 + 43 +
-# 2 x 152 = 461; 2-D (128^2): even 91 + 33 + 2 x 122 = 368, odd 79 + 33 + 2 x 122
-# = 356.  Set an entry to None whenever that kernel changes until it is re-captured.
-MEASURED_FP64_FLOP_PER_CELL = {2: 362.0, 3: 448.5}
+# the two parities.  3-D (128^3): even 60 + 19 + 2 x 141 = 361, odd 55 + 18 +
+# 2 x 146 = 365; 2-D (128^2): even 40 + 16 + 2 x 110 = 276, odd 38 + 16 + 2 x 112
+# = 278.  Set an entry to None whenever that kernel changes until it is re-captured.
+MEASURED_FP64_FLOP_PER_CELL = {2: 277.0, 3: 363.0}
 # FP64 pipe instructions (dadd + dmul + dfma) per cell update, mean of both parities, from the
 # same ncu capture: each takes one issue of the FP64 pipe, whose instruction rate is half the
 # measured FMA FLOP rate
-MEASURED_FP64_INSTR_PER_CELL = {2: 240.0, 3: 296.5}
-# the step kernel the roofline describes, per storage (3-D, nx % 8 == 0)
-STEP_KERNEL = {"f32": "k_ideal_step<3,float,float> (fused collide+stream)",
+MEASURED_FP64_INSTR_PER_CELL = {2: 166.0, 3: 219.5}
+# the step kernels the roofline describes, per storage (3-D, nx % 8 == 0)
+STEP_KERNEL = {"f32": "k_ideal_double<8> (two fused collide+stream steps a pass), k_ideal_step<3,float,float> "
+                      "where a run's steps do not fill a pair of passes",
                "f64": "k_ideal_step<3,double,double> (fused collide+stream; FP64-pipe bound on GB300)",
                "f16dev": "k_ideal_step_pairs<__half> (fused collide+stream, bulk-copy loads, 2 cells/thread)",
                "bf16dev": "k_ideal_step_pairs<__nv_bfloat16> (fused collide+stream, bulk-copy loads, 2 cells/thread)"}
@@ -313,12 +316,15 @@ def powell_form(args, vlbm, fields, torch, stream, hbm_peak):
     del Q, f0
     vlbm.vlbm_step(ctx.ptr, 4)
     steps = args.form_steps
+    l0 = ctx.launches
     ms = _time_steps(vlbm, [ctx.ptr], stream, torch, steps, False)
+    launches = ctx.launches - l0
     status = vlbm.status_string(vlbm.vlbm_sync(ctx.ptr))
     ctx.close()
     ncell = n ** 3
     gl = ncell * steps / (ms * 1e-3) / 1e9
-    bytes_cell = 2 * 63 * 4
+    # every launch reads and writes each population once; a two-step pass is one launch
+    bytes_cell = 2 * 63 * 4 * launches / steps
     return {"workload": "ideal MHD 3-D with the Powell source, %d^3, 9 x D3Q7 (the 8 fields and the "
                         "divergence lattice D), FP32, tau 0.51, tau_d 0.51, tau_M 1, same fields as the "
                         "headline workload, D = 0 at start" % n,
@@ -553,7 +559,10 @@ def batch_form(args, vlbm, fields, torch, stream, hbm_peak):
         bad += vlbm.vlbm_init_fields_device(bctx.ptr, d, Q.data_ptr()) != vlbm.VLBM_OK
     choice = bctx.autotune(8)
     vlbm.vlbm_step(bctx.ptr, 64)
+    l0 = bctx.launches
     ms_b = _time_steps(vlbm, [bctx.ptr], stream, torch, steps, False)
+    # every launch reads and writes each population once; a two-step pass is one launch
+    bytes_cell = 320 * (bctx.launches - l0) / steps
     st_b = vlbm.status_string(vlbm.vlbm_sync(bctx.ptr))
     # which domains left the physical states (NaN, rho <= 0 or p <= 0) by the end of the run:
     # the health flag is one per context; the cost of a step does not depend on the values
@@ -592,7 +601,7 @@ def batch_form(args, vlbm, fields, torch, stream, hbm_peak):
                     "(a context refuses steps after the flag is seen), so the baseline's rate is an upper "
                     "bound and the speedup a lower one",
             "nonphysical_cell_share": sum(side * side for _, side, _ in bad_domains) / ncell,
-            "bytes_per_cell": 320, "roofline_frac_batched": gb * 1e9 * 320 / (hbm_peak * 1e9)}
+            "bytes_per_cell": bytes_cell, "roofline_frac_batched": gb * 1e9 * bytes_cell / (hbm_peak * 1e9)}
 
 
 def ideal_2d_f64_form(args, vlbm, fields, torch, stream, fp64_tflops):
@@ -914,8 +923,15 @@ def main():
     # whole-job rate: every rank's cells over the slowest rank's time
     glups, ms_max, _ = vdist.weak_scaling_rate(ms, ncell, args.steps, device="cuda")
     bytes_cell = 2 * 56 * BYTES_PER_POP[args.storage]
-    per_launch_ms = ms / args.steps
+    # a two-step pass is one launch; a slab's launches include its halo copies
+    per_launch_ms = ms / (launches if world == 1 else args.steps)
     achieved = ncell * bytes_cell / (per_launch_ms * 1e-3) / 1e9
+    # launches that advanced two steps, and the mean DRAM bytes per cell of a launch
+    doubles = args.steps - launches if world == 1 else 0
+    dram_cell = MEASURED_DRAM_BYTES_PER_CELL.get(args.storage)
+    if dram_cell and doubles > 0:
+        two = MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS.get(args.storage)
+        dram_cell = ((launches - doubles) * dram_cell + doubles * two) / launches if two else None
     step_ms = ms_max / args.steps
     # spread: five more timed regions of the same length (every rank takes part in
     # the barriers; rank 0 reports its own; the line's value is the first region,
@@ -1046,7 +1062,8 @@ def main():
         scale = Q.reshape(8, -1).abs().amax(1)
         for form in ["f32"] + [f for f in form_list if f not in ("f64", "f32")]:
             c = make_ctx(form)
-            msf, _ = timed(c, nfs, 0, collective=False)
+            msf, lf = timed(c, nfs, 0, collective=False)
+            bf = 2 * 56 * BYTES_PER_POP[form] * lf / nfs  # each launch moves every population once
             Qf = moments_dev(c)
             st = vlbm.vlbm_sync(c.ptr)
             c.close()
@@ -1055,8 +1072,8 @@ def main():
             l2 = (diff.pow(2).mean(1).sqrt() / scale).cpu().numpy()
             del Qf, diff
             gl = ncell * nfs / (msf * 1e-3) / 1e9
-            forms[form] = {"glups": gl, "steps": nfs, "bytes_per_cell": 2 * 56 * BYTES_PER_POP[form],
-                           "roofline_frac": gl * 1e9 * 2 * 56 * BYTES_PER_POP[form] / (hbm_peak * 1e9),
+            forms[form] = {"glups": gl, "steps": nfs, "bytes_per_cell": bf,
+                           "roofline_frac": gl * 1e9 * bf / (hbm_peak * 1e9),
                            "status": vlbm.status_string(st),
                            "rel_linf_vs_f64": dict(zip(fields.IDEAL_FIELDS, [float(v) for v in linf])),
                            "rel_l2_vs_f64": dict(zip(fields.IDEAL_FIELDS, [float(v) for v in l2]))}
@@ -1113,8 +1130,8 @@ def main():
             "status": vlbm.status_string(status),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak,
-                         "traffic": (MEASURED_DRAM_BYTES_PER_CELL[args.storage] * ncell
-                                     if MEASURED_DRAM_BYTES_PER_CELL.get(args.storage) else None),
+                         "traffic": dram_cell * ncell if dram_cell else None,
+                         "two_step_launches": doubles,
                          "peak_kind": peak_kind,
                          "kernel": STEP_KERNEL[args.storage],
                          "algorithmic_bytes_per_launch": ncell * bytes_cell},
