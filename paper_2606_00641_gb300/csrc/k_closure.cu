@@ -1065,7 +1065,7 @@ __global__ void __launch_bounds__(256) k_part_sums(const __grid_constant__ PartS
 // 8 issues the MMAs).  While the MMAs run, warps 0-7 also sum the staged
 // output gradients per channel: the bias gradient.  Each CTA writes one
 // partial [cout][CIN][27] weight gradient followed by its [cout] bias
-// gradient (the parameter order), summed in fixed order by k_part_sum.
+// gradient (the parameter order), summed in fixed order by k_part_sums.
 constexpr int kWgZ = 2;
 constexpr int kWgThreads = 288;  // warps 0-7 stage, warp 8 issues the MMAs, warps 0-2 drain
 constexpr int kWgStage = 256;
