@@ -626,6 +626,11 @@ vlbm_status vlbm_step(vlbm_ctx *c, int n)
     // steps), and the launches outside graphs take one single step and then passes:
     // 512^3, 20 steps from step 5: 8.86 -> 7.31 ms a step.
     const int odd = (int)(c->step & 1);
+    // Launches of one call may be chained (launch_step_kernel), except under the caller's own
+    // capture, whose dependencies are the caller's, and on the default streams.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    c->chain = graphs && cudaStreamIsCapturing(c->stream, &capture) == cudaSuccess &&
+               capture == cudaStreamCaptureStatusNone;
     if ((odd && graphs ? n % kGraphLen : n) >= 4 + odd) ensure_second_buffer(c);
     int left = n;
     while (left > 0) {
@@ -1032,6 +1037,7 @@ vlbm_status vlbm_slabs_step(vlbm_ctx *const *slabs, int nslabs, int n)
     for (int t = 0; t < n; ++t) {
         for (int r = 0; r < nslabs; ++r) {
             vlbm_ctx *c = slabs[r];
+            c->chain = false;
             vlbm_status s = launch_step(c, (int)(c->step & 1));
             if (s != VLBM_OK) return s;
             c->step += 1;

@@ -95,6 +95,30 @@ inline StepGrid step_grid(int nx, int ny, int nz)
     else g.grid = dim3((unsigned)((nx + kBlockX - 1) / kBlockX), (unsigned)ny, (unsigned)nz);
     return g;
 }
+// Launch of a step kernel; chained: it may overlap the end of the launch before it
+// (programmatic dependent launch).  Its CTAs are set up as the previous step's last ones
+// leave, and wait in chain_wait() for that whole step and its writes before they touch
+// memory.  For steps of a few microseconds, where the gap between launches counts.
+template <class A>
+void launch_step_kernel(bool chained, void (*kernel)(A), dim3 grid, unsigned threads, cudaStream_t stream, const A &a)
+{
+    cudaLaunchAttribute chain = {};
+    chain.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    chain.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cfg.attrs = &chain;
+    cfg.numAttrs = chained;
+    cudaLaunchKernelEx(&cfg, kernel, a);  // its error is the caller's next cudaGetLastError
+}
+// The first statement of such a kernel that every thread with work reaches.
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
 // Calls f with the two run-time choices as compile-time ones.
 template <class F> void with_flags(bool first, bool second, F f)
 {
@@ -390,6 +414,7 @@ struct vlbm_ctx {
     void *double_doms = nullptr, *double_tiles = nullptr;  // 2-D: its constants and strip table
     int double_ntiles = 0;
     void *pop2 = nullptr;                // the two-step pass's other buffer (scratch between its two launches)
+    bool chain = false;                  // step launches of the current call may be chained (launch_step_kernel)
     bool pop2_tried = false;
     cudaEvent_t ev_copy[2]{}, ev_kern[2]{};  // per staging buffer: last copy / last kernel done
     cudaEvent_t flag_event = nullptr;
