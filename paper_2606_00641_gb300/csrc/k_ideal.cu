@@ -12,7 +12,9 @@
 // a few hundred flops per cell against 448 B at FP32/D3Q7), so the design
 // goal is plain bandwidth: one cell per thread, coalesced x-contiguous slot
 // planes, every load issued before any arithmetic, no shared memory, grid
-// (ceil(nx/128), ny, nz).
+// (ceil(nx/128), ny, nz), or CTAs along the cells of a plane where 128 does not divide nx.
+// Large plain FP32 3-D boxes take two steps per pass over the populations
+// (k_ideal_double), the only way left below one read and one write per step.
 #include <algorithm>
 
 #include "ideal_cell.cuh"
