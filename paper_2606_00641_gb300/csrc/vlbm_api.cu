@@ -238,14 +238,15 @@ void ensure_second_buffer(vlbm_ctx *c)
         return;
     }
     c->pop2_tried = true;
+    // the program may be capturing another stream in global mode, which an allocation in this
+    // thread would end; nothing here touches that capture
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     size_t avail = 0, total = 0;
-    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
-    if (c->pop_bytes > total / 6 || c->pop_bytes > avail / 3) return;
-    if (c->dim == 2 && double_2d_prepare(c) != VLBM_OK) return;
-    c->pop2 = dev_alloc(c, c->pop_bytes);
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) cudaGetLastError();
+    else if (c->pop_bytes <= total / 6 && c->pop_bytes <= avail / 3 && (c->dim == 3 || double_2d_prepare(c) == VLBM_OK))
+        c->pop2 = dev_alloc(c, c->pop_bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 // Launches the next of `left` steps from `parity`: four at once by two two-step passes,
