@@ -150,7 +150,7 @@ bool double_2d_ok(vlbm_ctx *c)
     return c->double_slots > 0;
 }
 
-// The strip table and the domains' constants on the device, once per context.
+// The strip table and the domains' constants on the device, when the context is created.
 vlbm_status double_2d_prepare(vlbm_ctx *c)
 {
     std::vector<StripDomain> doms;

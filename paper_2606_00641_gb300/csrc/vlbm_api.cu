@@ -244,8 +244,7 @@ void ensure_second_buffer(vlbm_ctx *c)
     cudaThreadExchangeStreamCaptureMode(&mode);
     size_t avail = 0, total = 0;
     if (cudaMemGetInfo(&avail, &total) != cudaSuccess) cudaGetLastError();
-    else if (c->pop_bytes <= total / 6 && c->pop_bytes <= avail / 3 && (c->dim == 3 || double_2d_prepare(c) == VLBM_OK))
-        c->pop2 = dev_alloc(c, c->pop_bytes);
+    else if (c->pop_bytes <= total / 6 && c->pop_bytes <= avail / 3) c->pop2 = dev_alloc(c, c->pop_bytes);
     cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
@@ -426,6 +425,12 @@ vlbm_status create_common(const vlbm_params *p, int count, vlbm_ctx **out)
         }
     }
     if (s == VLBM_OK && c->batched) s = batch_prepare(c);
+    // 2-D two-step passes: their strip table now, so that no step waits for its upload; without it
+    // every step is a launch of its own
+    if (s == VLBM_OK && c->dim == 2 && double_2d_ok(c) && double_2d_prepare(c) != VLBM_OK) {
+        c->double_slots = -1;
+        c->err.clear();
+    }
     if (s == VLBM_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "create synchronise");
     if (s != VLBM_OK) {
         g_err = c->err;

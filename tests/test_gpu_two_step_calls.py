@@ -48,3 +48,46 @@ def test_first_step_leaves_another_streams_capture_alone(V, shape):
         graph.replay()
         torch.cuda.synchronize()
         assert x.unique().tolist() == [2.0]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_first_step_does_not_wait_for_the_stream(V, shape):
+    import torch
+    with context(V, shape) as warm:
+        assert warm.step(4) == V.VLBM_OK and warm.sync() == V.VLBM_OK
+    side = torch.cuda.Stream()
+    with context(V, shape, stream=side.cuda_stream) as ctx:
+        done = torch.cuda.Event()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(2_000_000_000)  # about a second
+        before = ctx.launches
+        t = time.perf_counter()
+        assert ctx.step(4) == V.VLBM_OK
+        took = time.perf_counter() - t
+        done.record(side)
+        assert not done.query() and took < 0.3
+        assert ctx.sync() == V.VLBM_OK and ctx.launches - before == 2
+
+
+def test_refused_strip_table_takes_single_steps_and_leaves_no_error(V):
+    import torch
+    shape = (2048, 2048)
+    base = V.TorchHooks()
+    asked = []
+
+    def alloc(nbytes, stream, user):
+        asked.append(nbytes)
+        return base.alloc(nbytes, stream, user) if len(asked) != 3 else None  # populations, status block, table
+
+    class Hooks:
+        dealloc = base.dealloc
+
+    Hooks.alloc = V.ALLOC_FN(alloc)
+    Q = fields.uniform_ideal_state(shape, rho=1.1, u=(0.01, 0.02, 0.0), p=0.02, B=(0.01, 0.0, 0.02), gamma=1.5)
+    Qd = torch.as_tensor(Q, device="cuda")
+    with V.Context(V.make_params(shape=shape, storage="f32", gamma=1.5, tau=0.6, hooks=Hooks)) as ctx:
+        assert V.vlbm_init_fields_device(ctx.ptr, 0, Qd.data_ptr()) == V.VLBM_OK
+        before = ctx.launches
+        assert ctx.step(8) == V.VLBM_OK and ctx.sync() == V.VLBM_OK
+        assert ctx.launches - before == 8 and len(asked) >= 3
+        assert V.last_error(ctx.ptr) == ""
