@@ -204,9 +204,19 @@ vlbm_status vlbm_init_fields_device(vlbm_ctx *ctx, int domain, const double *Q_d
  * of vlbm_population_bytes (kept until vlbm_destroy), if the populations are at
  * most a sixth of the device's memory and a third of what is free; without it,
  * or on a stream under capture that has none yet, every step is one kernel.
+ * vlbm_set_two_step turns the passes off and gives that buffer back.
  * Returns the sticky status from the last health flag read back (a NaN,
  * rho <= 0 or p <= 0 seen by a step kernel gives VLBM_ERR_NONPHYSICAL). */
 vlbm_status vlbm_step(vlbm_ctx *ctx, int n);
+
+/* The two-step passes of vlbm_step off (on = 0) or on again (the default).  Off:
+ * the second population buffer, if there is one, is given back before the call
+ * returns (it waits for the stream; allocator hooks without a release keep it to
+ * vlbm_destroy), none is taken, and every later step is one kernel -- for a
+ * program that needs the memory, or the tile shape it chose, more than the speed.
+ * The populations are the same bit for bit.  Contexts that take no such passes
+ * accept the call. */
+vlbm_status vlbm_set_two_step(vlbm_ctx *ctx, int on);
 
 /* Wait for the context's stream and return the health status. */
 vlbm_status vlbm_sync(vlbm_ctx *ctx);
@@ -288,7 +298,8 @@ vlbm_status vlbm_load(vlbm_ctx *ctx, const void *buf, size_t bytes);
 /* Batched contexts: time each built tile configuration for `steps` steps on
  * the current state (state is restored afterwards) and keep the fastest;
  * *choice receives its index.  Single-domain contexts return VLBM_OK with
- * *choice = 0. */
+ * *choice = 0.  The choice is that of the kernel which advances one step: large
+ * batches take most steps two at a time (vlbm_step, vlbm_set_two_step). */
 vlbm_status vlbm_autotune(vlbm_ctx *ctx, int steps, int *choice);
 
 /* ------------------------------------------------------------------------
@@ -506,7 +517,7 @@ vlbm_status vlbm_slabs_step(vlbm_ctx *const *slabs, int nslabs, int n);
 
 /* Batched contexts: number of built tile shapes, and explicit selection of
  * one (0 <= shape < vlbm_tile_shapes; VLBM_ERR_ARG otherwise).  Single-domain
- * contexts have 0 shapes. */
+ * contexts have 0 shapes.  For the kernel of one step, as in vlbm_autotune. */
 int vlbm_tile_shapes(const vlbm_ctx *ctx);
 vlbm_status vlbm_set_tile_shape(vlbm_ctx *ctx, int shape);
 
@@ -541,7 +552,8 @@ int vlbm_num_domains(const vlbm_ctx *ctx);
 int64_t vlbm_num_cells(const vlbm_ctx *ctx, int domain);
 int64_t vlbm_step_count(const vlbm_ctx *ctx);
 int64_t vlbm_launch_count(const vlbm_ctx *ctx);      /* kernels this ctx launched */
-size_t vlbm_population_bytes(const vlbm_ctx *ctx);   /* device bytes of populations */
+size_t vlbm_population_bytes(const vlbm_ctx *ctx);   /* device bytes of populations (without the second
+                                                        buffer that vlbm_step may take) */
 void *vlbm_stream(const vlbm_ctx *ctx);              /* the cudaStream_t in use */
 const char *vlbm_last_error(const vlbm_ctx *ctx);
 const char *vlbm_status_string(int status);

@@ -47,14 +47,27 @@ void *dev_alloc(vlbm_ctx *c, size_t bytes)
     return p;
 }
 
+void dev_release(vlbm_ctx *c, const std::pair<void *, size_t> &pr)
+{
+    if (c->params.dealloc)
+        c->params.dealloc(pr.first, pr.second, (void *)c->stream, c->params.alloc_user);
+    else if (!c->params.alloc)
+        cudaFree(pr.first);
+}
+
+void dev_free(vlbm_ctx *c, void *p)
+{
+    for (size_t i = 0; i < c->owned.size(); ++i)
+        if (c->owned[i].first == p) {
+            dev_release(c, c->owned[i]);
+            c->owned.erase(c->owned.begin() + (std::ptrdiff_t)i);
+            return;
+        }
+}
+
 void dev_free_all(vlbm_ctx *c)
 {
-    for (auto &pr : c->owned) {
-        if (c->params.dealloc)
-            c->params.dealloc(pr.first, pr.second, (void *)c->stream, c->params.alloc_user);
-        else if (!c->params.alloc)
-            cudaFree(pr.first);
-    }
+    for (auto &pr : c->owned) dev_release(c, pr);
     c->owned.clear();
 }
 
@@ -227,7 +240,7 @@ vlbm_status launch_step(vlbm_ctx *c, int parity)
 // memory is plentiful: populations of at most a sixth of the device's memory, with at least
 // twice that much free beside it.  Without it (or while the stream is being captured by
 // the caller, when nothing may be allocated) every step is a launch of its own.
-bool double_ok(vlbm_ctx *c) { return c->dim == 3 ? ideal_double_ok(c) : double_2d_ok(c); }
+bool double_ok(vlbm_ctx *c) { return c->two_step && (c->dim == 3 ? ideal_double_ok(c) : double_2d_ok(c)); }
 
 void ensure_second_buffer(vlbm_ctx *c)
 {
@@ -1074,6 +1087,23 @@ vlbm_status vlbm_slabs_step(vlbm_ctx *const *slabs, int nslabs, int n)
     }
     for (int r = 0; r < nslabs; ++r) schedule_check(slabs[r], n);
     return c0->sticky;
+}
+
+vlbm_status vlbm_set_two_step(vlbm_ctx *c, int on)
+{
+    if (!c) return VLBM_ERR_ARG;
+    if (c->two_step == (on != 0)) return VLBM_OK;
+    drop_graphs(c);  // captured steps hold the passes and the second buffer
+    c->two_step = on != 0;
+    // given back at once, unless the allocator hooks have no release; and tried again once on
+    if (!on && c->pop2 && (c->params.dealloc || !c->params.alloc)) {
+        vlbm_status s = cuda_check(c, cudaStreamSynchronize(c->stream), "stream synchronise");
+        if (s != VLBM_OK) return s;
+        dev_free(c, c->pop2);
+        c->pop2 = nullptr;
+    }
+    c->pop2_tried = c->pop2 != nullptr;
+    return VLBM_OK;
 }
 
 int vlbm_tile_shapes(const vlbm_ctx *c) { return (c && c->batched) ? batch_num_choices() : 0; }

@@ -416,6 +416,7 @@ struct vlbm_ctx {
     void *pop2 = nullptr;                // the two-step pass's other buffer (scratch between its two launches)
     bool chain = false;                  // step launches of the current call may be chained (launch_step_kernel)
     bool pop2_tried = false;
+    bool two_step = true;                // vlbm_set_two_step
     cudaEvent_t ev_copy[2]{}, ev_kern[2]{};  // per staging buffer: last copy / last kernel done
     cudaEvent_t flag_event = nullptr;
     bool flag_pending = false;

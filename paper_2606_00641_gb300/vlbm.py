@@ -132,6 +132,7 @@ def load(build: bool = True):
         "vlbm_init_fields_f32": (i, [P, i, P]),
         "vlbm_moments_f32": (i, [P, i, P]),
         "vlbm_step": (i, [P, i]),
+        "vlbm_set_two_step": (i, [P, i]),
         "vlbm_sync": (i, [P]),
         "vlbm_moments": (i, [P, i, P]),
         "vlbm_moments_device": (i, [P, i, P]),
@@ -352,6 +353,10 @@ def vlbm_step(ctx: int, n: int) -> int:
     if st not in (VLBM_OK, VLBM_ERR_NONPHYSICAL, VLBM_ERR_TIMEOUT):
         _check(st, "vlbm_step", ctx)
     return st
+
+
+def vlbm_set_two_step(ctx: int, on: bool = True):
+    _check(load().vlbm_set_two_step(ctx, int(on)), "vlbm_set_two_step", ctx)
 
 
 def vlbm_sync(ctx: int) -> int:
@@ -670,6 +675,10 @@ class Context:
 
     def step(self, n: int) -> int:
         return vlbm_step(self.ptr, n)
+
+    def set_two_step(self, on: bool = True) -> None:
+        """Allow or refuse the two-step passes and their second buffer; see ``vlbm_set_two_step``."""
+        vlbm_set_two_step(self.ptr, on)
 
     def sync(self) -> int:
         return vlbm_sync(self.ptr)

@@ -91,3 +91,50 @@ def test_refused_strip_table_takes_single_steps_and_leaves_no_error(V):
         assert ctx.step(8) == V.VLBM_OK and ctx.sync() == V.VLBM_OK
         assert ctx.launches - before == 8 and len(asked) >= 3
         assert V.last_error(ctx.ptr) == ""
+
+
+@pytest.mark.parametrize("hooked", [False, True])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_two_step_off_gives_the_memory_back(V, shape, hooked):
+    import torch
+    cells = np.random.default_rng(1).integers(0, int(np.prod(shape)), 100000)
+    f0 = fields.ideal_fields(shape, 23, mach=0.5, beta=1.0, cfl=0.1, device=torch.device("cuda"))
+    base, held = V.TorchHooks(), {}
+
+    def alloc(nbytes, stream, user):
+        p = base.alloc(nbytes, stream, user)
+        held[p] = nbytes
+        return p
+
+    def dealloc(ptr, nbytes, stream, user):
+        assert held.pop(ptr) == nbytes
+        base.dealloc(ptr, nbytes, stream, user)
+
+    class Hooks:
+        pass
+
+    Hooks.alloc, Hooks.dealloc = V.ALLOC_FN(alloc), V.FREE_FN(dealloc)
+    got = []
+    for switched in (False, True):
+        p = V.make_params(shape=shape, storage="f32", gamma=f0.gamma, tau=0.6, hooks=Hooks if hooked else None)
+        with V.Context(p) as ctx:
+            pops = V.vlbm_population_bytes(ctx.ptr)
+            assert V.vlbm_init_fields_device(ctx.ptr, 0, f0.Q.data_ptr()) == V.VLBM_OK
+            marks = [ctx.launches]
+            for n, on in ((40, True), (40, False), (7, False), (8, True)):
+                if switched:
+                    ctx.set_two_step(on)
+                assert ctx.step(n) == V.VLBM_OK and ctx.sync() == V.VLBM_OK
+                marks.append(ctx.launches)
+                if switched:
+                    free = torch.cuda.mem_get_info()[0]
+                    ctx.set_two_step(False)
+                    if hooked:
+                        assert list(held.values()).count(pops) == 1
+                    elif on:
+                        assert torch.cuda.mem_get_info()[0] - free >= pops
+            passes = np.diff(marks).tolist()
+            # from step 87 (odd): a single step, a pass of four, three single steps
+            assert passes == ([20, 40, 7, 6] if switched else [20, 20, 5, 6])
+            got.append(ctx.populations(cells))
+    assert np.array_equal(got[0], got[1]) and not held
