@@ -77,8 +77,8 @@ template <class C, bool SWAP> __device__ __forceinline__ constexpr int slot_orde
 }
 
 // Steps that may be chained (launch_step_kernel): the plain FP32 ones.  150 x 200, 60 steps
-// with sums every 10: 500 -> 441 us; 64^2, 128 steps on three streams 116 -> 98 us; 128^2,
-// 64^3 and larger the same.  Not FP64, whose waiting CTAs were placed unevenly over the
+// with sums every 10: 500 -> 441 us; 64^2, 128 steps on three streams 116 -> 98 us; in graphs
+// where chain_in_graph says so.  Not FP64, whose waiting CTAs were placed unevenly over the
 // SMs: 128^2, 200 steps 1.87 -> 2.34 ms.  HOM reads its fields by the read-only path.
 template <class S, class C, bool CORR, bool HOM>
 constexpr bool kChained = sizeof(C) == 4 && !Codec<S>::kDev && !CORR && !HOM;

@@ -547,7 +547,7 @@ vlbm_status resistive_step(vlbm_ctx *c, int parity)
     const StepGrid g = step_grid(d.nx, d.ny, d.nz);
     a.by_nx = g.nx;
     with_flags(parity != 0, g.planes, [&](auto odd, auto planes) {
-        // chained: 8 x 32 x 32, 100 steps 132 -> 113 us; 20 x 50 x 60 267 -> 257 us; larger the same
+        // chained: 8 x 32 x 32, 100 steps 132 -> 113 us; 20 x 50 x 60 267 -> 257 us
         launch_step_kernel(c->chain, k_res_step<decltype(odd)::value, decltype(planes)::value>, g.grid, kBlockX,
                            c->stream, a);
     });
