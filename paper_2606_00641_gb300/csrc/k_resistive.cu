@@ -226,19 +226,23 @@ __global__ void __launch_bounds__(kBlockX, 5) k_res_step(const Args a)
         }
 }
 
-// f = f_eq(rho, m - F/2, B), g = g_eq(B, u = m/rho) at parity 0, rounded to FP32 once.
-// Carried in split floats (split_f32.cuh): in FP64, with the velocities in a table, the
-// pass took 4.22 ms at 128 x 128 x 256 for 0.13 ms worth of memory traffic; 0.49 ms so.  Opposite
-// directions share the part even in c, w (rho + 4.5 (c c - cs2 I):(rho v v + ...)), and
-// differ in the sign of the odd one, 3 w c.j.
+// f = f_eq(rho, m - F/2, B), g = g_eq(B, u = m/rho) at parity 0: the FP64 expressions' values
+// rounded to FP32 once.  Carried in split floats (split_f32.cuh): in FP64, with the velocities in
+// a table, the pass took 4.22 ms at 128 x 128 x 256 for 0.13 ms worth of memory traffic; 0.62-0.66 ms
+// so.  Opposite directions share the part even in c, w (rho + 4.5 (c c - cs2 I):(rho v v + ...)),
+// and differ in the sign of the odd one, 3 w c.j.  Split floats keep some 42 bits of the largest
+// term, so where a value lies that close to the middle of two floats (in one cell of some
+// two thousand) the population is formed again in FP64, and each is the FP64 form's.
 struct InitArgs {
     float *pop;
     int64_t stride, c0, count, qstride;
     double F[3];
 };
 
-// The same in FP64, for states beyond the range in which split floats keep their digits.
-__device__ __noinline__ void res_init_wide(const InitArgs &a, const double *__restrict__ Qin, int64_t t, float *out)
+// In FP64, the populations whose bits are set (flow, magnetic): all for states beyond the range in
+// which split floats keep their digits, else those next to a rounding boundary.
+__device__ __noinline__ void res_init_wide(const InitArgs &a, const double *__restrict__ Qin, int64_t t, float *out,
+                                           uint32_t flow, uint32_t magnetic)
 {
     const double rho = Qin[t];
     double m[3], j[3], B[3], u[3], v[3];
@@ -253,6 +257,7 @@ __device__ __noinline__ void res_init_wide(const InitArgs &a, const double *__re
     const double B2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
 #pragma unroll 1
     for (int i = 0; i < kQf; ++i) {
+        if (!((flow >> i) & 1u)) continue;
         const int c[3] = {cx19(i), cy19(i), cz19(i)};
         const double cv = c[0] * v[0] + c[1] * v[1] + c[2] * v[2];
         const double cj = c[0] * j[0] + c[1] * j[1] + c[2] * j[2];
@@ -264,6 +269,7 @@ __device__ __noinline__ void res_init_wide(const InitArgs &a, const double *__re
     }
 #pragma unroll 1
     for (int i = 0; i < 21; ++i) {
+        if (!((magnetic >> i) & 1u)) continue;
         const int b = i / 7, d = i % 7, ax = (d - 1) / 2;
         double cphi = 0.0;
         if (d > 0 && ax != b) cphi = ((d & 1) ? 1.0 : -1.0) * (u[ax] * B[b] - B[ax] * u[b]);
@@ -279,9 +285,12 @@ __global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double
     {
         bool usual = Qin[t] > 1e-6 && Qin[t] < 1e6;
 #pragma unroll
-        for (int k = 1; k < 7; ++k) usual = usual && fabs(Qin[k * a.qstride + t]) < 1e6;
+        for (int k = 1; k < 7; ++k) {
+            const double v = fabs(Qin[k * a.qstride + t]);
+            usual = usual && v < 1e6 && (v > 1e-30 || v == 0.0);
+        }
         if (!usual) {
-            res_init_wide(a, Qin, t, out);
+            res_init_wide(a, Qin, t, out, ~0u, ~0u);
             return;
         }
     }
@@ -296,6 +305,16 @@ __global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double
         u[ax] = split(m) * ir;
         v[ax] = j[ax] * ir;
     }
+    // Bounds of the errors below, u = 2^-24: a split input is off by u^2 of itself, a product by
+    // 6 u^2, a sum by 3 u^2, the reciprocal by 6 u^2 (its Newton step leaves (2 u)^2); so rho (c.v)^2 by
+    // 2^-42.9 of rho |v|_1^2, and a flow population by 2^-41.9 of w `most`; a magnetic one by 2^-43 of
+    // its terms.  Taken as 2^-41 and 2^-42, which covers the FP64 form's own 2^-50 and these
+    // sums' roundings too, and 2^-125 for what is lost below the normal floats (2^-149 a product,
+    // times a component of at most 2^20).
+    auto one_norm = [](const Split (&x)[3]) { return fabsf(x[0].hi) + fabsf(x[1].hi) + fabsf(x[2].hi); };
+    const float sv = one_norm(v), sB = one_norm(B);
+    const float most = rho.hi + 3.f * one_norm(j) + 6.1f * rho.hi * sv * sv + 8.3f * sB * sB;
+    uint32_t flow = 0u, magnetic = 0u;  // populations to form again
     const Split third = {1.f / 3.f, (float)(1.0 / 3.0 - (double)(1.f / 3.f))};
     const Split B2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
     const Split v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
@@ -321,16 +340,22 @@ __global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double
                 }
             return s;
         };
+        const float off = 0x1p-41f * w.hi * most;
         if (p == 0) {
-            out[0] = (w * (rho + four_half * (base - hB2))).hi;
+            const Split f = w * (rho + four_half * (base - hB2));
+            out[0] = f.hi;
+            if (!rounds_surely(f, off)) flow |= 1u;
             continue;
         }
         const Split cv = along(v), cB = along(B);
         Split second = base + rho * (cv * cv) - cB * cB;
         if (i > 6) second = second + hB2;
         const Split even = w * (rho + four_half * second), odd = w * (three * along(j));
-        out[(int64_t)i * a.stride] = (even + odd).hi;
-        out[(int64_t)(i + 1) * a.stride] = (even - odd).hi;
+        const Split plus = even + odd, minus = even - odd;
+        out[(int64_t)i * a.stride] = plus.hi;
+        out[(int64_t)(i + 1) * a.stride] = minus.hi;
+        if (!rounds_surely(plus, off)) flow |= 1u << i;
+        if (!rounds_surely(minus, off)) flow |= 2u << i;
     }
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
@@ -341,10 +366,17 @@ __global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double
         for (int ax = 0; ax < 3; ++ax) {  // w (B +- 4 (u_a B_b - B_a u_b)), zero for a = b
             Split s = {0.f, 0.f};
             if (ax != b) s = halfs * (u[ax] * B[b] - B[ax] * u[b]);
-            g[(int64_t)(2 * ax + 1) * a.stride] = (B8 + s).hi;
-            g[(int64_t)(2 * ax + 2) * a.stride] = (B8 - s).hi;
+            const Split plus = B8 + s, minus = B8 - s;
+            g[(int64_t)(2 * ax + 1) * a.stride] = plus.hi;
+            g[(int64_t)(2 * ax + 2) * a.stride] = minus.hi;
+            if (ax == b) continue;  // B / 8 itself, rounded once by the split
+            const float terms = fabsf(B8.hi) + 0.5f * (fabsf(u[ax].hi * B[b].hi) + fabsf(B[ax].hi * u[b].hi));
+            const float off = terms > 0.f ? fmaf(0x1p-42f, terms, 0x1p-125f) : 0.f;
+            if (!rounds_surely(plus, off)) magnetic |= 1u << (7 * b + 2 * ax + 1);
+            if (!rounds_surely(minus, off)) magnetic |= 2u << (7 * b + 2 * ax + 1);
         }
     }
+    if ((flow | magnetic) != 0u) res_init_wide(a, Qin, t, out, flow, magnetic);
 }
 
 struct ReadArgs {

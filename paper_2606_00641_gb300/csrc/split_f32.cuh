@@ -78,4 +78,10 @@ __device__ __forceinline__ Split reciprocal(Split a)
     return renorm(q, __fmul_rn(q, r));
 }
 
+// Whether a value within `off` (>= 0) of a rounds to a.hi whatever it is.
+__device__ __forceinline__ bool rounds_surely(Split a, float off)
+{
+    return __fadd_rn(a.hi, __fadd_ru(a.lo, off)) == a.hi && __fadd_rn(a.hi, __fsub_rd(a.lo, off)) == a.hi;
+}
+
 }  // namespace vlbm
