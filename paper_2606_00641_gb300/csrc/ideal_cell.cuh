@@ -200,7 +200,7 @@ VLBM_HD __forceinline__ void ideal_collide_f64(C (&f)[8][AxisSet<D>::Q], const C
 // relax: a function from lattice to its constants and source terms.  The two directions of an axis get
 // +- omega phi / 2 last, as one rounded value (see relax_lattice).
 template <int D, int NL = 8, class W>
-__device__ __forceinline__ void ideal_collide_f32(float (&f)[NL][AxisSet<D>::Q], const float gm1, const W &relax,
+VLBM_HD __forceinline__ void ideal_collide_f32(float (&f)[NL][AxisSet<D>::Q], const float gm1, const W &relax,
                                                   unsigned *flags, const float inv_tau_m = 0.f)
 {
     constexpr int Q = AxisSet<D>::Q;
@@ -209,20 +209,20 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[NL][AxisSet<D>::Q],
     for (int k = 0; k < NL; ++k) {
         float s = f[k][0];
 #pragma unroll
-        for (int i = 1; i < Q; ++i) s = __fadd_rn(s, f[k][i]);
+        for (int i = 1; i < Q; ++i) s = add_rn(s, f[k][i]);
         q[k] = s;
     }
-    const float ir = __frcp_rn(q[0]);
+    const float ir = rcp_rn(q[0]);
     const float m[3] = {q[1], q[2], q[3]}, B[3] = {q[5], q[6], q[7]};
-    const float u[3] = {__fmul_rn(m[0], ir), __fmul_rn(m[1], ir), __fmul_rn(m[2], ir)};
+    const float u[3] = {mul_rn(m[0], ir), mul_rn(m[1], ir), mul_rn(m[2], ir)};
     auto dot = [](const float (&a)[3], const float (&b)[3]) {
-        return __fmaf_rn(a[2], b[2], __fmaf_rn(a[1], b[1], __fmul_rn(a[0], b[0])));
+        return fma_rn(a[2], b[2], fma_rn(a[1], b[1], mul_rn(a[0], b[0])));
     };
     const float B2 = dot(B, B), uB = dot(u, B);
-    const float p = __fmul_rn(gm1, __fmaf_rn(-0.5f, B2, __fmaf_rn(-0.5f, dot(m, u), q[4])));
-    const float pt = __fmaf_rn(0.5f, B2, p);
+    const float p = mul_rn(gm1, fma_rn(-0.5f, B2, fma_rn(-0.5f, dot(m, u), q[4])));
+    const float pt = fma_rn(0.5f, B2, p);
     if (!(q[0] > 0.f) || !(p > 0.f)) raise_flag(flags, kFlagNonPhysical);
-    const float Ept = __fadd_rn(q[4], pt);
+    const float Ept = add_rn(q[4], pt);
     float phi[NL][D];
 #pragma unroll
     for (int ax = 0; ax < D; ++ax) {
@@ -233,39 +233,39 @@ __device__ __forceinline__ void ideal_collide_f32(float (&f)[NL][AxisSet<D>::Q],
                 phi[1 + b][ax] = phi[1 + ax][b];
                 phi[5 + b][ax] = -phi[5 + ax][b];
             } else {
-                const float t = __fmaf_rn(m[ax], u[b], -__fmul_rn(B[ax], B[b]));
-                phi[1 + b][ax] = ax == b ? __fadd_rn(t, pt) : t;
-                phi[5 + b][ax] = ax == b ? 0.f : __fmaf_rn(u[ax], B[b], -__fmul_rn(B[ax], u[b]));
+                const float t = fma_rn(m[ax], u[b], -mul_rn(B[ax], B[b]));
+                phi[1 + b][ax] = ax == b ? add_rn(t, pt) : t;
+                phi[5 + b][ax] = ax == b ? 0.f : fma_rn(u[ax], B[b], -mul_rn(B[ax], u[b]));
             }
         }
-        phi[4][ax] = __fmaf_rn(Ept, u[ax], -__fmul_rn(B[ax], uB));
+        phi[4][ax] = fma_rn(Ept, u[ax], -mul_rn(B[ax], uB));
     }
     float ndiv = 0.f;  // Powell form: -div B
     if constexpr (NL == 9) {
-        ndiv = __fmul_rn(-q[8], inv_tau_m);
+        ndiv = mul_rn(-q[8], inv_tau_m);
 #pragma unroll
-        for (int ax = 0; ax < D; ++ax) phi[8][ax] = __fmaf_rn(q[8], u[ax], -B[ax]);
+        for (int ax = 0; ax < D; ++ax) phi[8][ax] = fma_rn(q[8], u[ax], -B[ax]);
     }
 #pragma unroll
     for (int k = 0; k < NL; ++k) {
         const RelaxSource r = relax(k);
-        float A0 = __fmaf_rn(r.ow0, q[k], r.src0), A1 = __fmaf_rn(r.ow1, q[k], r.src1);
+        float A0 = fma_rn(r.ow0, q[k], r.src0), A1 = fma_rn(r.ow1, q[k], r.src1);
         if constexpr (NL == 9) {
             if (k > 0) {  // S = -(div B)(0, B, u.B, u) and, for D, -D / tau_M = -div B
                 const float S = k == 8   ? ndiv
-                                : k >= 5 ? __fmul_rn(ndiv, u[k >= 5 && k < 8 ? k - 5 : 0])
-                                : k == 4 ? __fmul_rn(ndiv, uB)
-                                         : __fmul_rn(ndiv, B[k >= 1 && k < 4 ? k - 1 : 0]);
-                A0 = __fmaf_rn(ExactWeights<D, float>::w0, S, A0);
-                A1 = __fmaf_rn(ExactWeights<D, float>::w1, S, A1);
+                                : k >= 5 ? mul_rn(ndiv, u[k >= 5 && k < 8 ? k - 5 : 0])
+                                : k == 4 ? mul_rn(ndiv, uB)
+                                         : mul_rn(ndiv, B[k >= 1 && k < 4 ? k - 1 : 0]);
+                A0 = fma_rn(ExactWeights<D, float>::w0, S, A0);
+                A1 = fma_rn(ExactWeights<D, float>::w1, S, A1);
             }
         }
-        f[k][0] = __fmaf_rn(r.omc, f[k][0], A0);
+        f[k][0] = fma_rn(r.omc, f[k][0], A0);
 #pragma unroll
         for (int ax = 0; ax < D; ++ax) {
-            const float bv = __fmul_rn(r.hom, phi[k][ax]);
-            f[k][2 * ax + 1] = __fadd_rn(__fmaf_rn(r.omc, f[k][2 * ax + 1], A1), bv);
-            f[k][2 * ax + 2] = __fsub_rn(__fmaf_rn(r.omc, f[k][2 * ax + 2], A1), bv);
+            const float bv = mul_rn(r.hom, phi[k][ax]);
+            f[k][2 * ax + 1] = add_rn(fma_rn(r.omc, f[k][2 * ax + 1], A1), bv);
+            f[k][2 * ax + 2] = sub_rn(fma_rn(r.omc, f[k][2 * ax + 2], A1), bv);
         }
     }
 }

@@ -243,6 +243,20 @@ template <int D, class C> VLBM_HD __forceinline__ Relax<C> relax_at(const C *ome
     return relax_of<D, C>(omega[k]);
 }
 
+// Single operations rounded to nearest, never fused or reordered; on the host (built without
+// contraction) the plain operators are that.
+#ifdef __CUDA_ARCH__
+#define VLBM_RN(device, host) device
+#else
+#define VLBM_RN(device, host) host
+#endif
+VLBM_HD __forceinline__ float add_rn(float a, float b) { return VLBM_RN(__fadd_rn(a, b), a + b); }
+VLBM_HD __forceinline__ float sub_rn(float a, float b) { return VLBM_RN(__fsub_rn(a, b), a - b); }
+VLBM_HD __forceinline__ float mul_rn(float a, float b) { return VLBM_RN(__fmul_rn(a, b), a * b); }
+VLBM_HD __forceinline__ float fma_rn(float a, float b, float c) { return VLBM_RN(__fmaf_rn(a, b, c), fmaf(a, b, c)); }
+VLBM_HD __forceinline__ float rcp_rn(float a) { return VLBM_RN(__frcp_rn(a), 1.f / a); }
+#undef VLBM_RN
+
 // Keep an FP64 value in registers: without it the compiler adds a cell's populations
 // up a second time for the relaxation, to hold fewer registers over the fluxes -- 32 of
 // 202 FP64 instructions a cell in 2-D, 44 of 271 in 3-D, on the pipe that binds those
