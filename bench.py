@@ -10,7 +10,8 @@ GLUPS (10^9 cell updates per second, whole job) and the fraction of the HBM
 roofline (448 algorithmic bytes per cell and launch: every population read once
 and written once).
 
-Printed: one JSON line on rank 0.  ``--impl reference`` times the CPU oracle
+Printed: one JSON line on rank 0 (the full record, with every form, sweep and path, goes
+to standard error).  ``--impl reference`` times the CPU oracle
 (plain FP64 C) on the host cores on a bounded sample of the same workload.
 Under torchrun (N > 1) the ranks hold the z-slabs of one periodic domain of
 512 x 512 x (512 N) cells, one 512^3 slab per rank (the 512^3 fields repeated
@@ -823,6 +824,28 @@ def compact_summary(line):
     return out
 
 
+def printed_line(line):
+    """The line on standard output: the headline with its workload, roofline, clocks and
+    end-to-end figure, and one [GLUPS, fraction] per other path -- short enough for a reader
+    who keeps the last couple of kilobytes.  The full record goes to standard error."""
+    def only(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else None
+
+    out = {k: v for k, v in line.items()
+           if k not in ("config", "roofline", "clocks", "repeats", "slab_check", "e2e", "cpu_baseline", "forms",
+                        "error_growth", "other_paths", "paper_context", "summary")}
+    out["config"] = only(line["config"], "workload", "grid", "storage", "parallelism", "l2")
+    out["roofline"] = only(line["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic")
+    out["clocks"] = line["clocks"]
+    out["e2e"] = only(line["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    if line.get("slab_check"):
+        out["slab_check"] = line["slab_check"]
+    out["cpu_baseline"] = only(line.get("cpu_baseline"), "value", "unit", "cores")
+    out["paths"] = {k: v[:2] for k, v in line["summary"].items()
+                    if k != "headline" and isinstance(v, list) and v and all(isinstance(x, float) for x in v[:2])}
+    return out
+
+
 def main():
     args = parse()
     world, rank, local = dist_env()
@@ -1149,7 +1172,8 @@ def main():
             "fp64_tflops": fp64_tflops,
         }
         line["summary"] = compact_summary(line)
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(printed_line(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
     return 0
