@@ -42,11 +42,11 @@ BYTES_PER_POP = {"f64": 8, "f32": 4, "f16dev": 2, "bf16dev": 2}
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of a 256^3 launch of
 # each parity, mean of the two parities, taken after the last change to that
 # kernel's source: f32 7,457,546 kB and f16dev 3,703,464 kB per 16,777,216-cell
-# launch, and 8,004,037 kB per two-step pass (f32).  Traffic grows in proportion to the cells, so a full launch is this
-# times the cells.  Set an entry to None whenever that kernel changes until it
-# is re-captured.
+# launch, which at another size grows in proportion to the cells; and f32 8,004,037 kB
+# per two-step pass at 256^3, which need not.  Set an entry to None whenever that
+# kernel changes until it is re-captured.
 MEASURED_DRAM_BYTES_PER_CELL = {"f32": 7457546e3 / 16777216, "f16dev": 3703464e3 / 16777216}
-MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS = {"f32": 8004037e3 / 16777216}
+MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS = {("f32", 256): 8004037e3 / 16777216}
 # FP64 operations per cell update of the FP64 step kernels (k_ideal_step<D,double>),
 # from one ncu capture of each parity: (dadd + dmul + 2 dfma thread instructions,
 # smsp__sass_thread_inst_executed_op_d{add,mul,fma}_pred_on.sum) / cells, mean of
@@ -824,6 +824,18 @@ def compact_summary(line):
     return out
 
 
+def dram_bytes_per_cell(storage, n, launches, doubles):
+    """Mean DRAM bytes per cell of a launch, `doubles` of `launches` advancing two steps, or None
+    where it is not measured.  A single step's traffic is in proportion to the cells; a two-step
+    pass re-reads rims from L2 in part, more or less of them with the box and the height of its
+    columns, so its figure stands for the box it was captured on alone."""
+    one = MEASURED_DRAM_BYTES_PER_CELL.get(storage)
+    if not doubles or one is None:
+        return one
+    two = MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS.get((storage, n))
+    return ((launches - doubles) * one + doubles * two) / launches if two else None
+
+
 def printed_line(line):
     """The line on standard output: the headline with its workload, roofline, clocks and
     end-to-end figure, and one [GLUPS, fraction] per other path -- short enough for a reader
@@ -951,10 +963,7 @@ def main():
     achieved = ncell * bytes_cell / (per_launch_ms * 1e-3) / 1e9
     # launches that advanced two steps, and the mean DRAM bytes per cell of a launch
     doubles = args.steps - launches if world == 1 else 0
-    dram_cell = MEASURED_DRAM_BYTES_PER_CELL.get(args.storage)
-    if dram_cell and doubles > 0:
-        two = MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS.get(args.storage)
-        dram_cell = ((launches - doubles) * dram_cell + doubles * two) / launches if two else None
+    dram_cell = dram_bytes_per_cell(args.storage, n, launches, doubles)
     step_ms = ms_max / args.steps
     # spread: five more timed regions of the same length (every rank takes part in
     # the barriers; rank 0 reports its own; the line's value is the first region,

@@ -1,4 +1,4 @@
-"""The line that the benchmark prints: every key of the headline, and short -- a reader of the
+"""The line that the benchmark prints (and the DRAM figures in it): every key of the headline, and short -- a reader of the
 last two kilobytes of output has it whole."""
 import json
 
@@ -43,3 +43,13 @@ def test_printed_line_without_end_to_end():
     line = dict(full_line(), e2e=None, cpu_baseline=None)
     out = bench.printed_line(line)
     assert out["e2e"] is None and out["cpu_baseline"] is None
+
+
+def test_traffic_of_two_step_passes_only_at_the_size_it_was_captured():
+    one = bench.MEASURED_DRAM_BYTES_PER_CELL["f32"]
+    two = bench.MEASURED_DRAM_BYTES_PER_CELL_TWO_STEPS["f32", 256]
+    assert bench.dram_bytes_per_cell("f32", 512, 20, 0) == one
+    assert bench.dram_bytes_per_cell("f32", 512, 10, 10) is None
+    assert bench.dram_bytes_per_cell("f32", 256, 10, 10) == two
+    assert abs(bench.dram_bytes_per_cell("f32", 256, 11, 9) - (2 * one + 9 * two) / 11) < 1e-9
+    assert bench.dram_bytes_per_cell("f64", 512, 20, 0) is None
