@@ -1319,10 +1319,8 @@ struct LossArgs {
 // r = (Q1 - Qt)/sigma, loss += sum r^2 / N, gq = 2 r / (sigma N).  blockIdx.y = field.
 // The FP64 pipe binds it, so an element takes three FP64 operations and two conversions
 // (the weights per field come from the host, 1/sigma^2 is applied to the field's sum) and
-// a CTA reduces by shuffles; before, each element was divided by N, multiplied three times by
+// a CTA (one per SM and field) reduces by shuffles; before, each element was divided by N, multiplied three times by
 // 1/sigma or 2/N, and 1216 CTAs took a 255-addition tree each: 36 -> 24 us at 64^3.
-constexpr int kLossBlocks = 152;
-
 __global__ void __launch_bounds__(256) k_loss(const double *__restrict__ q1, const double *__restrict__ qt, int N,
                                               const LossArgs la, float *__restrict__ gq, double *__restrict__ loss)
 {
@@ -1938,7 +1936,7 @@ vlbm_status loss_backward(vlbm_closure *cl, const double *Qt_dev, cudaStream_t s
             la.g[k] = (double)(2.0f / (float)cl->N) * inv * inv;
         }
         la.inv_n = 0.5 * (double)(2.0f / (float)cl->N);
-        const unsigned blocks = (unsigned)std::min((cl->N + 255) / 256, kLossBlocks);
+        const unsigned blocks = (unsigned)std::min((cl->N + 255) / 256, cl->sms);
         k_loss<<<dim3(blocks, 8), 256, 0, s>>>(cl->q1, Qt_dev, cl->N, la, cl->gq, cl->loss);
         k_grad_out<<<(cl->N + 255) / 256, 256, 0, s>>>(cl->gq, cl->nx, cl->ny, cl->nz, cl->col_scale, cl->gy);
         st = cl_check(cudaGetLastError(), "closure loss launch");
