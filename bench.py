@@ -854,7 +854,7 @@ def printed_line(line):
         out["slab_check"] = line["slab_check"]
     out["cpu_baseline"] = only(line.get("cpu_baseline"), "value", "unit", "cores")
     out["paths"] = {k: v[:2] for k, v in line["summary"].items()
-                    if k != "headline" and isinstance(v, list) and v and all(isinstance(x, float) for x in v[:2])}
+                    if k != "headline" and "_err_" not in k and isinstance(v, list) and v and all(isinstance(x, float) for x in v[:2])}
     return out
 
 

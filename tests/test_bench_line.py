@@ -21,7 +21,7 @@ def full_line():
                       "l2": "inputs_larger_than_l2 (30.1 GB of populations per rank)"}
     line["roofline"] = {"bound": "hbm", "achieved": 4934.123456789, "peak": 6784.2, "unit": "GB/s",
                         "frac": 0.727312345678, "traffic": None, "kernel": bench.STEP_KERNEL["f32"]}
-    line["summary"] = bench.compact_summary(line)
+    line["summary"] = dict(bench.compact_summary(line), channel_u_err_5000=[0.6, 0.3, 0.08])
     return line
 
 
@@ -36,6 +36,7 @@ def test_printed_line_is_short_and_whole():
     assert out["e2e"] == {k: line["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")}
     assert out["roofline"]["frac"] == line["roofline"]["frac"]
     assert out["paths"]["form_f16dev"] == [27.0, 0.9] and out["paths"]["channel"] == [20.5, 0.98]
+    assert not any("_err_" in k for k in out["paths"])  # rates only
     assert json.loads(json.dumps(out)) == out
 
 
