@@ -1570,9 +1570,10 @@ vlbm_status conv(vlbm_closure *cl, int layer, const bf16 *in, bool transpose, co
         // tcgen05 / TMEM columns of 8 x 16 cells: persistent CTAs, one per SM.  A CTA of few
         // slices spends most of its time on the weights' copy and the two planes a run adds,
         // so up to 64 CTAs each takes what there is and beyond that at least four slices.
-        // 32^3 (256 slices), 128 steps: 4.13 ms on 152 CTAs and 4.46 on 64 when alone, 2.96
-        // and 1.96 a run when three contexts share the GPU; 16^3 (32 slices): 3.63 ms on 32
-        // CTAs, 4.18 on 8.
+        // Microseconds a step of a closure run, alone / three contexts at once, with this rule and
+        // with min(slices, SMs) CTAs: 64 slices 28.6 / 33.7 both; 128: 29.7 / 37.5 and 29.3 / 54.4;
+        // 192: 32.6 / 41.3 and 31.3 / 66.0; 256 (32^3): 34.9 / 44.9 and 31.7 / 65.9; 384: 36.5 / 62.4
+        // and 34.9 / 77.6; 512: 37.6 / 80.9 and 37.9 / 89.0; from 608 the same.
         const int64_t slices = (int64_t)(cl->nx / kTcX) * (cl->ny / kTcY) * cl->nz;
         const unsigned grid = (unsigned)std::min<int64_t>({slices, cl->sms, std::max<int64_t>(64, slices / 4)});
         const int cout_real = transpose ? kCin[layer] : kCout[layer];
