@@ -336,9 +336,9 @@ void drop_graphs(vlbm_ctx *c)
 // they pile up on some SMs.  Measured in CTAs per SM, graphs of 32 steps, plain / chained:
 //   2-D      2.95 1.13   3.4 0.85   4.6 0.93   5.3 1.02   (and 1.37 .. 1.9: 0.93 .. 1.00)
 //   2-D Powell  2.95 1.13   3.4 0.89   4.2 0.99   4.6 1.02
-//   3-D      2.3 1.15   2.6 0.81   4.0 0.94   4.2 1.07
+//   3-D      2.4 1.11   2.6 0.81   4.0 0.94   4.2 1.07
 //   3-D Powell  2.0 1.12   2.1 0.87   3.0 0.97   4.0 1.08   (and 1.37 .. 1.9: 0.89 .. 0.94)
-//   channel  2.3 1.11   2.6 0.83   4.0 1.00   4.2 1.10
+//   channel  2.4 1.11   2.6 0.83   4.0 1.00   4.2 1.10
 bool chain_in_graph(const vlbm_ctx *c)
 {
     int dev = 0, sms = 0;
@@ -352,7 +352,7 @@ bool chain_in_graph(const vlbm_ctx *c)
     const double each = (double)g.x * g.y * g.z / sms;
     const bool powell = c->nlat == 9, uneven = each > 1.3 && each < 2.0;
     if (c->dim == 2) return powell ? each <= 3.0 || each > 4.4 : !uneven && (each <= 3.0 || each > 5.1);
-    return powell ? !uneven && (each <= 2.0 || each >= 4.0) : each < 2.35 || each > 4.05;
+    return powell ? !uneven && (each <= 2.0 || each >= 4.0) : each <= 2.5 || each > 4.05;
 }
 
 cudaGraphExec_t get_graph(vlbm_ctx *c, int parity, int len, int64_t *launches)
