@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kBlockX, 5) k_res_step(const Args a)
 
 // f = f_eq(rho, m - F/2, B), g = g_eq(B, u = m/rho) at parity 0: the FP64 expressions' values
 // rounded to FP32 once.  Carried in split floats (split_f32.cuh): in FP64, with the velocities in
-// a table, the pass took 4.22 ms at 128 x 128 x 256 for 0.13 ms worth of memory traffic; 0.62-0.66 ms
+// a table, the pass took 4.22 ms at 128 x 128 x 256 for 0.13 ms worth of memory traffic; 0.53-0.54 ms
 // so.  Opposite directions share the part even in c, w (rho + 4.5 (c c - cs2 I):(rho v v + ...)),
 // and differ in the sign of the odd one, 3 w c.j.  Split floats keep some 42 bits of the largest
 // term, so where a value lies that close to the middle of two floats (in one cell of some
@@ -240,40 +240,51 @@ struct InitArgs {
 };
 
 // In FP64, the populations whose bits are set (flow, magnetic): all for states beyond the range in
-// which split floats keep their digits, else those next to a rounding boundary.
+// which split floats keep their digits, else the one or two next to a rounding boundary, for
+// which nothing is formed that they do not need (the whole cell: 0.65 against 0.54 ms at
+// 128 x 128 x 256, and 41 against 36 us at 46 x 19 x 24, where a pass is a wave or two).
 __device__ __noinline__ void res_init_wide(const InitArgs &a, const double *__restrict__ Qin, int64_t t, float *out,
                                            uint32_t flow, uint32_t magnetic)
 {
     const double rho = Qin[t];
-    double m[3], j[3], B[3], u[3], v[3];
-    for (int ax = 0; ax < 3; ++ax) {
-        m[ax] = Qin[(1 + ax) * a.qstride + t];
-        B[ax] = Qin[(4 + ax) * a.qstride + t];
-        j[ax] = m[ax] - 0.5 * a.F[ax];
-        u[ax] = m[ax] / rho;
-        v[ax] = j[ax] / rho;
+    const double *m = Qin + a.qstride + t, *B = Qin + 4 * a.qstride + t;
+    if (flow) {
+        double j[3], v[3], b[3];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            j[ax] = m[ax * a.qstride] - 0.5 * a.F[ax];
+            v[ax] = j[ax] / rho;
+            b[ax] = B[ax * a.qstride];
+        }
+        const double v2 = (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) / 3.0;
+        const double B2 = b[0] * b[0] + b[1] * b[1] + b[2] * b[2];
+        for (; flow; flow &= flow - 1u) {
+            const int i = __ffs((int)flow) - 1;
+            const int c[3] = {cx19(i), cy19(i), cz19(i)};
+            double cv = 0.0, cj = 0.0, cB = 0.0;
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax)
+                if (c[ax] != 0) {
+                    cv += c[ax] > 0 ? v[ax] : -v[ax];
+                    cj += c[ax] > 0 ? j[ax] : -j[ax];
+                    cB += c[ax] > 0 ? b[ax] : -b[ax];
+                }
+            // B^2 (c^2 - 1) / 2 + B^2 / 3 for c^2 = 0, 1, 2
+            const double even = i == 0 ? -1.0 / 6.0 : (i <= 6 ? 1.0 / 3.0 : 5.0 / 6.0);
+            const double second = rho * (cv * cv - v2) + (even * B2 - cB * cB);
+            const double w = i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
+            out[(int64_t)i * a.stride] = (float)(w * (rho + 3.0 * cj + 4.5 * second));
+        }
     }
-    const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    const double B2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
-#pragma unroll 1
-    for (int i = 0; i < kQf; ++i) {
-        if (!((flow >> i) & 1u)) continue;
-        const int c[3] = {cx19(i), cy19(i), cz19(i)};
-        const double cv = c[0] * v[0] + c[1] * v[1] + c[2] * v[2];
-        const double cj = c[0] * j[0] + c[1] * j[1] + c[2] * j[2];
-        const double cB = c[0] * B[0] + c[1] * B[1] + c[2] * B[2];
-        const double c2 = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
-        const double second = rho * (cv * cv - v2 / 3.0) + 0.5 * B2 * (c2 - 1.0) - (cB * cB - B2 / 3.0);
-        const double w = i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
-        out[(int64_t)i * a.stride] = (float)(w * (rho + 3.0 * cj + 4.5 * second));
-    }
-#pragma unroll 1
-    for (int i = 0; i < 21; ++i) {
-        if (!((magnetic >> i) & 1u)) continue;
-        const int b = i / 7, d = i % 7, ax = (d - 1) / 2;
+    for (; magnetic; magnetic &= magnetic - 1u) {
+        const int i = __ffs((int)magnetic) - 1, k = i / 7, d = i % 7, ax = (d - 1) / 2;
+        const double Bk = B[k * a.qstride];
         double cphi = 0.0;
-        if (d > 0 && ax != b) cphi = ((d & 1) ? 1.0 : -1.0) * (u[ax] * B[b] - B[ax] * u[b]);
-        out[(int64_t)(kQf + i) * a.stride] = (float)((d == 0 ? 0.25 : 0.125) * (B[b] + 4.0 * cphi));
+        if (d > 0 && ax != k) {
+            cphi = m[ax * a.qstride] / rho * Bk - B[ax * a.qstride] * (m[k * a.qstride] / rho);
+            if (!(d & 1)) cphi = -cphi;
+        }
+        out[(int64_t)(kQf + i) * a.stride] = (float)((d == 0 ? 0.25 : 0.125) * (Bk + 4.0 * cphi));
     }
 }
 
@@ -283,14 +294,18 @@ __global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double
     if (t >= a.count) return;
     float *out = a.pop + a.c0 + t;
     {
-        bool usual = Qin[t] > 1e-6 && Qin[t] < 1e6;
+        // rho in 2^-19 .. 2^19, components zero or 2^-99 .. 2^19 in size: on the upper words, as
+        // each comparison in FP64 takes 16 cycles of an SM
+        auto word = [](double x) { return (uint32_t)__double2hiint(x); };
+        auto exponent = [](int e) { return (uint32_t)(1023 + e) << 20; };
+        bool usual = word(Qin[t]) >= exponent(-19) && word(Qin[t]) < exponent(19);
 #pragma unroll
         for (int k = 1; k < 7; ++k) {
-            const double v = fabs(Qin[k * a.qstride + t]);
-            usual = usual && v < 1e6 && (v > 1e-30 || v == 0.0);
+            const uint32_t v = word(Qin[k * a.qstride + t]) & 0x7FFFFFFFu;
+            usual = usual && v < exponent(19) && (v >= exponent(-99) || v == 0u);
         }
         if (!usual) {
-            res_init_wide(a, Qin, t, out, ~0u, ~0u);
+            res_init_wide(a, Qin, t, out, (1u << kQf) - 1u, (1u << 21) - 1u);
             return;
         }
     }
@@ -310,7 +325,7 @@ __global__ void __launch_bounds__(128) k_res_init(const InitArgs a, const double
     // 2^-42.9 of rho |v|_1^2, and a flow population by 2^-41.9 of w `most`; a magnetic one by 2^-43 of
     // its terms.  Taken as 2^-41 and 2^-42, which covers the FP64 form's own 2^-50 and these
     // sums' roundings too, and 2^-125 for what is lost below the normal floats (2^-149 a product,
-    // times a component of at most 2^20).
+    // times a component below 2^19).
     auto one_norm = [](const Split (&x)[3]) { return fabsf(x[0].hi) + fabsf(x[1].hi) + fabsf(x[2].hi); };
     const float sv = one_norm(v), sB = one_norm(B);
     const float most = rho.hi + 3.f * one_norm(j) + 6.1f * rho.hi * sv * sv + 8.3f * sB * sB;
