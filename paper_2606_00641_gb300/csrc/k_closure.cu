@@ -375,8 +375,8 @@ __device__ __forceinline__ bool tc_wait(uint32_t mb, uint32_t phase, volatile in
     return false;
 }
 
-// The same without parking: for a hand-over between two threads that is a few dozen
-// cycles away (a parked thread takes some hundred cycles to come back).
+// The same without parking: for the hand-over between the two issuing threads (a parked
+// thread takes some hundred cycles to come back).
 __device__ __forceinline__ bool tc_spin(uint32_t mb, uint32_t phase, volatile int *abort)
 {
     for (uint32_t it = 0; it < 256u; ++it) {
@@ -492,9 +492,10 @@ __device__ __forceinline__ void tc_plane(uint32_t hb, uint32_t d, uint64_t w, ui
 // The three z-taps are stacked along N: halo plane h (2-D tap (dx, dy), K-chunk j)
 // times [W(dz=0) | W(dz=1) | W(dz=2)] (N = 96) contributes to the output slices h, h-1
 // and h-2 at once, whose accumulators lie in consecutive 32-column blocks (tc_slot;
-// where the ring of blocks wraps, two MMAs).  An M128 K16 MMA costs about 60 cycles for
-// any N up to 96, and the MMA issue binds: so each plane is read and multiplied once,
-// 18 MMAs (Cin = 32) a slice plus two planes a run.  Measured (launch list) against tiles
+// where the ring of blocks wraps, two MMAs: two planes in sixteen).  An M128 K16 MMA costs
+// about 60 cycles for any N up to 96, so it is their number that counts: each plane is
+// read and multiplied once, 18 MMAs (Cin = 32) a slice, 20 with the wrap, plus two planes a
+// run.  At 128^3 the tensor pipe is 44 % active, 95 cycles an MMA.  Measured (launch list) against tiles
 // of four slices, which multiplied six planes for four slices: Cin = 32 at 128^3 130 -> 107
 // us, at 64^3 33 -> 22; Cin = 8 at 128^3 64 -> 59 us, at 64^3 18 -> 14.  With one issuing
 // thread, whose waits and descriptors cost some 800 cycles a plane, 132 us at 128^3; with

@@ -118,8 +118,9 @@ int strip_width(int nx)
 
 // Where the pass is taken: 2-D FP32 domains that together exceed L2, with strips that fill
 // the device: of the cells that all waves of warps could produce, rims and end rows
-// included, at least 0.6 are wanted cells.  The gain is proportional to that share: 1.56 for
-// the 64 domains above (0.79), 1.44 at 1000^2 (0.76).
+// included, at least 0.6 are wanted cells.  The gain is proportional to that share: 1.60 for
+// the 64 domains above (0.79), 1.44 at 1000^2 (0.76).  Eleven other domains, 920^2 .. 4096^2, thin ones
+// among them: 1.34 .. 1.48; six batches of equal domains 64^2 .. 600^2: 1.48 .. 1.58.
 bool double_2d_ok(vlbm_ctx *c)
 {
     if (c->model != VLBM_IDEAL || c->nlat != 8 || c->dim != 2 || c->storage != VLBM_F32 || c->slab || c->closure ||

@@ -1175,7 +1175,9 @@ template <int NL> static int double_slots_of_device()
 // Where the two-step pass is taken: plain (or Powell) 3-D FP32 boxes whose populations
 // exceed L2 (below, a step is not bound by HBM) and whose columns fill the CTA slots well,
 // a share of at least 0.7.  The gain is proportional to the share: 1.27 at 512^3 (0.84),
-// 1.17 at 128^3 (0.71), 0.91 at 96^3 (0.45); Powell 90 x 130 x 150 (0.80) 1.28.
+// 1.17 at 128^3 (0.71), 0.91 at 96^3 (0.45); Powell 90 x 130 x 150 (0.80) 1.28.  Against single
+// steps, 32 steps: 15 plain boxes taken, 110^3 .. 302^3 and 16 x 512^2 among them, 1.17 .. 1.36 (1.21 to
+// 1.25 at shares of 0.71 .. 0.79); nine Powell boxes, 110^3 .. 256^3, shares 0.76 .. 0.87, 1.12 .. 1.29.
 bool ideal_double_ok(vlbm_ctx *c)
 {
     if (c->batched || (c->model != VLBM_IDEAL && c->model != VLBM_IDEAL_POWELL) || c->dim != 3 ||
