@@ -211,11 +211,12 @@ vlbm_status vlbm_step(vlbm_ctx *ctx, int n);
 
 /* The two-step passes of vlbm_step off (on = 0) or on again (the default).  Off:
  * the second population buffer, if there is one, is given back before the call
- * returns (it waits for the stream; allocator hooks without a release keep it to
- * vlbm_destroy), none is taken, and every later step is one kernel -- for a
- * program that needs the memory, or the tile shape it chose, more than the speed.
- * The populations are the same bit for bit.  Contexts that take no such passes
- * accept the call. */
+ * returns (it waits for the stream; kept to vlbm_destroy where the allocator
+ * hooks have no release, or where the caller has captured steps that use it), none
+ * is taken, and every later step is one kernel -- for a program that needs the
+ * memory, or the tile shape it chose, more than the speed.  The populations are
+ * the same bit for bit.  Contexts that take no such passes accept the call.
+ * VLBM_ERR_STATE: a buffer to give back while the stream is being captured. */
 vlbm_status vlbm_set_two_step(vlbm_ctx *ctx, int on);
 
 /* Wait for the context's stream and return the health status. */

@@ -678,9 +678,11 @@ vlbm_status vlbm_step(vlbm_ctx *c, int n)
     // Launches of one call may be chained (launch_step_kernel), except under the caller's own
     // capture, whose dependencies are the caller's, and on the default streams.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    c->chain = graphs && cudaStreamIsCapturing(c->stream, &capture) == cudaSuccess &&
-               capture == cudaStreamCaptureStatusNone;
+    const bool known = cudaStreamIsCapturing(c->stream, &capture) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    c->chain = graphs && known && capture == cudaStreamCaptureStatusNone;
     if ((odd && graphs ? n % kGraphLen : n) >= 4 + odd) ensure_second_buffer(c);
+    if (capture != cudaStreamCaptureStatusNone) c->pop2_captured = c->pop2_captured || c->pop2 != nullptr;
     int left = n;
     while (left > 0) {
         if (graphs && left >= kGraphLen) {
@@ -1123,15 +1125,24 @@ vlbm_status vlbm_set_two_step(vlbm_ctx *c, int on)
 {
     if (!c) return VLBM_ERR_ARG;
     if (c->two_step == (on != 0)) return VLBM_OK;
-    drop_graphs(c);  // captured steps hold the passes and the second buffer
-    c->two_step = on != 0;
-    // given back at once, unless the allocator hooks have no release; and tried again once on
-    if (!on && c->pop2 && (c->params.dealloc || !c->params.alloc)) {
+    // given back at once, unless the allocator hooks have no release or a graph that the caller
+    // captured holds it; and tried again once on
+    if (!on && c->pop2 && !c->pop2_captured && (c->params.dealloc || !c->params.alloc)) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return fail(c, VLBM_ERR_STATE, "two-step passes: not while the stream is being captured");
+        }
         vlbm_status s = cuda_check(c, cudaStreamSynchronize(c->stream), "stream synchronise");
         if (s != VLBM_OK) return s;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // as in ensure_second_buffer
+        cudaThreadExchangeStreamCaptureMode(&mode);
         dev_free(c, c->pop2);
+        cudaThreadExchangeStreamCaptureMode(&mode);
         c->pop2 = nullptr;
     }
+    drop_graphs(c);  // captured steps hold the passes and the second buffer
+    c->two_step = on != 0;
     c->pop2_tried = c->pop2 != nullptr;
     return VLBM_OK;
 }

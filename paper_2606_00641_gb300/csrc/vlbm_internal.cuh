@@ -431,6 +431,7 @@ struct vlbm_ctx {
     bool chain = false;                  // step launches of the current call may be chained (launch_step_kernel)
     bool pop2_tried = false;
     bool two_step = true;                // vlbm_set_two_step
+    bool pop2_captured = false;          // a graph of the caller's may hold pop2
     cudaEvent_t ev_copy[2]{}, ev_kern[2]{};  // per staging buffer: last copy / last kernel done
     cudaEvent_t flag_event = nullptr;
     bool flag_pending = false;

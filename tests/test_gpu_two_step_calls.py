@@ -138,3 +138,49 @@ def test_two_step_off_gives_the_memory_back(V, shape, hooked):
             assert passes == ([20, 40, 7, 6] if switched else [20, 20, 5, 6])
             got.append(ctx.populations(cells))
     assert np.array_equal(got[0], got[1]) and not held
+
+
+def test_two_step_off_keeps_what_a_callers_graph_holds(V):
+    import torch
+    shape = (128, 128, 128)
+    cells = np.random.default_rng(1).integers(0, int(np.prod(shape)), 100000)
+    f0 = fields.ideal_fields(shape, 23, mach=0.5, beta=1.0, cfl=0.1, device=torch.device("cuda"))
+    got = []
+    for captured in (False, True):
+        side = torch.cuda.Stream()
+        p = V.make_params(shape=shape, storage="f32", gamma=f0.gamma, tau=0.6, stream=side.cuda_stream)
+        with V.Context(p) as ctx:
+            assert V.vlbm_init_fields_device(ctx.ptr, 0, f0.Q.data_ptr()) == V.VLBM_OK
+            assert ctx.step(4) == V.VLBM_OK
+            if captured:
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=side):
+                    assert ctx.step(8) == V.VLBM_OK
+                free = torch.cuda.mem_get_info()[0]
+                ctx.set_two_step(False)
+                assert torch.cuda.mem_get_info()[0] - free < V.vlbm_population_bytes(ctx.ptr)
+                other = torch.full((V.vlbm_population_bytes(ctx.ptr),), 7, dtype=torch.uint8, device="cuda")
+                with torch.cuda.stream(side):
+                    graph.replay()
+                torch.cuda.synchronize()
+                assert bool((other == 7).all())
+            else:
+                assert ctx.step(8) == V.VLBM_OK
+            assert ctx.sync() == V.VLBM_OK and ctx.step_count == 12
+            got.append(ctx.populations(cells))
+    assert np.array_equal(got[0], got[1])
+
+
+def test_two_step_off_is_refused_under_capture(V):
+    import torch
+    side = torch.cuda.Stream()
+    with context(V, (128, 128, 128), stream=side.cuda_stream) as ctx:
+        assert ctx.step(4) == V.VLBM_OK and ctx.sync() == V.VLBM_OK
+        graph = torch.cuda.CUDAGraph()
+        x = torch.zeros(10, device="cuda")
+        with torch.cuda.graph(graph, stream=side):
+            x.add_(1)
+            with pytest.raises(V.VlbmError):
+                ctx.set_two_step(False)
+        before = ctx.launches
+        assert ctx.step(4) == V.VLBM_OK and ctx.sync() == V.VLBM_OK and ctx.launches - before == 2
