@@ -77,8 +77,7 @@ template <class C, bool SWAP> __device__ __forceinline__ constexpr int slot_orde
 }
 
 // Steps that may be chained (launch_step_kernel): the plain FP32 ones.  150 x 200, 60 steps
-// with sums every 10: 500 -> 441 us; 64^2, 128 steps on three streams 116 -> 98 us; in graphs
-// where chain_in_graph says so.  Not FP64, whose waiting CTAs were placed unevenly over the
+// with sums every 10: 500 -> 441 us; 64^2, 128 steps on three streams 116 -> 98 us.  Not FP64, whose waiting CTAs were placed unevenly over the
 // SMs: 128^2, 200 steps 1.87 -> 2.34 ms.  HOM reads its fields by the read-only path.
 template <class S, class C, bool CORR, bool HOM>
 constexpr bool kChained = sizeof(C) == 4 && !Codec<S>::kDev && !CORR && !HOM;
@@ -156,6 +155,7 @@ __device__ __forceinline__ void ideal_step_body(const IdealArgs<C> &a)
             const int64_t at = ODD ? nb[i] : cell;
             Codec<S>::store(pop + (int64_t)(k * Q + j) * a.stride + at, f[k][i]);
         }
+    if constexpr (kChained<S, C, CORR, HOM>) chain_next();
 }
 
 template <int D, class S, class C, bool ODD, bool PLANES, bool CORR = false, int NL = 8, bool HOM = false>

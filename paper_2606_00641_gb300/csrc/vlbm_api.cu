@@ -328,33 +328,6 @@ void drop_graphs(vlbm_ctx *c)
     c->graph_launches.clear();
 }
 
-// Whether the steps of a captured graph are chained (launch_step_kernel).  Launched one by
-// one, chained steps were never slower (32 to 1216 CTAs a step: 1.09 to 2.0 times as fast,
-// the host binds).  In a graph the gap between plain steps is small already, and what counts
-// is where the waiting CTAs are placed: evenly where those of two steps fit the SMs
-// together, or where a step fills the SMs and its CTAs follow as others leave; in between
-// they pile up on some SMs.  Measured in CTAs per SM, graphs of 32 steps, plain / chained:
-//   2-D      2.95 1.13   3.4 0.85   4.6 0.93   5.3 1.02   (and 1.37 .. 1.9: 0.93 .. 1.00)
-//   2-D Powell  2.95 1.13   3.4 0.89   4.2 0.99   4.6 1.02
-//   3-D      2.4 1.11   2.6 0.81   4.0 0.94   4.2 1.07
-//   3-D Powell  2.0 1.12   2.1 0.87   3.0 0.97   4.0 1.08   (and 1.37 .. 1.9: 0.89 .. 0.94)
-//   channel  2.4 1.11   2.6 0.83   4.0 1.00   4.2 1.10
-bool chain_in_graph(const vlbm_ctx *c)
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-        cudaGetLastError();
-        return false;
-    }
-    const Domain &d = c->dom[0];
-    const dim3 g = step_grid(d.nx, d.ny, d.nz).grid;
-    const double each = (double)g.x * g.y * g.z / sms;
-    const bool powell = c->nlat == 9, uneven = each > 1.3 && each < 2.0;
-    if (c->dim == 2) return powell ? each <= 3.0 || each > 4.4 : !uneven && (each <= 3.0 || each > 5.1);
-    return powell ? !uneven && (each <= 2.0 || each >= 4.0) : each <= 2.5 || each > 4.05;
-}
-
 cudaGraphExec_t get_graph(vlbm_ctx *c, int parity, int len, int64_t *launches)
 {
     const int key = parity * 1024 + len;
@@ -368,12 +341,9 @@ cudaGraphExec_t get_graph(vlbm_ctx *c, int parity, int len, int64_t *launches)
         return nullptr;
     }
     const int64_t before = c->launches;
-    const bool chain = c->chain;
-    c->chain = chain && chain_in_graph(c);
     bool ok = true;
     for (int s = 0, taken = 0; s < len && ok; s += taken)
         ok = launch_next(c, parity == 0, (parity + s) & 1, len - s, &taken) == VLBM_OK;
-    c->chain = chain;
     const int64_t captured = c->launches - before;
     c->launches = before;
     cudaGraph_t g = nullptr;
@@ -441,6 +411,10 @@ vlbm_status create_common(const vlbm_params *p, int count, vlbm_ctx **out)
         s = cuda_check(c, cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking), "stream create");
         c->own_stream = s == VLBM_OK;
     }
+    int dev = 0;
+    if (s == VLBM_OK) s = cuda_check(c, cudaGetDevice(&dev), "device query");
+    if (s == VLBM_OK)
+        s = cuda_check(c, cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev), "device query");
     if (s == VLBM_OK) s = cuda_check(c, cudaEventCreateWithFlags(&c->flag_event, cudaEventDisableTiming),
                                      "event create");
     if (s == VLBM_OK) s = cuda_check(c, cudaMallocHost(&c->h_flags, kStatusBytes), "pinned flag word");

@@ -96,9 +96,14 @@ inline StepGrid step_grid(int nx, int ny, int nz)
     return g;
 }
 // Launch of a step kernel; chained: it may overlap the end of the launch before it
-// (programmatic dependent launch).  Its CTAs are set up as the previous step's last ones
-// leave, and wait in chain_wait() for that whole step and its writes before they touch
-// memory.  For steps of a few microseconds, where the gap between launches counts.
+// (programmatic dependent launch).  Its CTAs are set up once all of the previous step's are
+// past their stores (chain_next), and wait in chain_wait() for that whole step and its writes
+// before they touch memory.  For steps of a few microseconds, where the gap between
+// launches counts.  Let in earlier, at the previous step's start, the waiting CTAs took
+// whatever room was left and piled up on some SMs: graphs of 32 steps of 1.4 .. 1.9 or 2.5 .. 5
+// CTAs per SM were up to 23 per cent slower than plain ones (2-D 256^2 3.8 -> 4.5 us a step);
+// let in at the end they are 1.04 to 1.24 times as fast as plain ones at every size from 32
+// to 1216 CTAs, plain 2-D, Powell, 3-D and channel steps alike (256^2: 3.4 us).
 template <class A>
 void launch_step_kernel(bool chained, void (*kernel)(A), dim3 grid, unsigned threads, cudaStream_t stream, const A &a)
 {
@@ -113,12 +118,9 @@ void launch_step_kernel(bool chained, void (*kernel)(A), dim3 grid, unsigned thr
     cfg.numAttrs = chained;
     cudaLaunchKernelEx(&cfg, kernel, a);  // its error is the caller's next cudaGetLastError
 }
-// The first statement of such a kernel that every thread with work reaches.
-__device__ __forceinline__ void chain_wait()
-{
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
+// The first statement of such a kernel that every thread with work reaches, and its last.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 // Calls f with the two run-time choices as compile-time ones.
 template <class F> void with_flags(bool first, bool second, F f)
 {
@@ -422,6 +424,7 @@ struct vlbm_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaStream_t copy_stream = nullptr;  // host-field staging copies (overlap the chunk kernels)
+    int sms = 0;                         // streaming multiprocessors of the device
     int bulk_ctas = 0;                   // persistent grid of the bulk-load step (0: not sized yet)
     int double_slots = 0;                // CTAs (2-D: strips) of the two-step pass that the device holds
                                          // (0: not asked yet, -1: the pass is not taken)
