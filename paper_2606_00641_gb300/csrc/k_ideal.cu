@@ -77,8 +77,9 @@ template <class C, bool SWAP> __device__ __forceinline__ constexpr int slot_orde
 }
 
 // Steps that may be chained (launch_step_kernel): the plain FP32 ones.  150 x 200, 60 steps
-// with sums every 10: 500 -> 441 us; 64^2, 128 steps on three streams 116 -> 98 us.  Not FP64, whose waiting CTAs were placed unevenly over the
-// SMs: 128^2, 200 steps 1.87 -> 2.34 ms.  HOM reads its fields by the read-only path.
+// with sums every 10: 500 -> 395 us; other sizes beside launch_step_kernel.  Not FP64: let in
+// at the step's start, its waiting CTAs were placed unevenly over the SMs (128^2, 200 steps
+// 1.87 -> 2.34 ms; not measured with the end).  HOM reads its fields by the read-only path.
 template <class S, class C, bool CORR, bool HOM>
 constexpr bool kChained = sizeof(C) == 4 && !Codec<S>::kDev && !CORR && !HOM;
 
